@@ -314,15 +314,15 @@ __global__ void k_nesterov_plain(const float* __restrict__ reg, const float2* __
 // Twiddle table of the length-n transform with forward radices r[0..s) in
 // direction D (the inverse runs them reversed), in the layout the stage
 // runner reads: stage k >= 1 of radix R after NS points holds W^(q j), q =
-// 1..R-1, j < NS, at (sum of (R_i - 1) NS_i over the stages 1..k-1) + (q - 1)
-// NS + j; computed in double precision and rounded once.
+// 1..R-1, j < NS, at (sum of tw_size over the stages 1..k-1) + tw_entry(NS, q,
+// j); computed in double precision and rounded once.
 bool host_twiddles_radices(int n, const int* r, int s, int D, std::vector<float2>& tab) {
   auto radix = [&](int k) { return D == FWD ? r[k] : r[s - 1 - k]; };
   int prod = 1;
   for (int k = 0; k < s; k++) prod *= radix(k);
   if (prod != n) return false;
   size_t len = 0;
-  for (int k = 1, ns = radix(0); k < s; ns *= radix(k), k++) len += (size_t)(radix(k) - 1) * ns;
+  for (int k = 1, ns = radix(0); k < s; ns *= radix(k), k++) len += tw_size(radix(k), ns);
   tab.assign(len > 0 ? len : 1, make_float2(1.f, 0.f));
   size_t off = 0;
   for (int k = 1, ns = radix(0); k < s; ns *= radix(k), k++) {
@@ -331,16 +331,16 @@ bool host_twiddles_radices(int n, const int* r, int s, int D, std::vector<float2
       for (int j = 0; j < ns; j++) {
         const long m = ((long)q * j) % ((long)ns * R);
         const double ang = 2.0 * M_PI * (double)m / (double)(ns * R);
-        tab[off + (size_t)(q - 1) * ns + j] = make_float2((float)std::cos(ang), (float)(D * std::sin(ang)));
+        tab[off + tw_entry(ns, q, j)] = make_float2((float)std::cos(ang), (float)(D * std::sin(ang)));
       }
-    off += (size_t)(R - 1) * ns;
+    off += tw_size(R, ns);
   }
   return true;
 }
 
 // Twiddle table of the length-n transform in direction D, in the layout the
 // stage runner reads (stage k >= 1 of radix R after NS points: W^(r j) at
-// stage_twoff + (r - 1) NS + j), computed in double precision.
+// stage_twoff + tw_entry(NS, r, j)), computed in double precision.
 bool host_twiddles(int n, int D, std::vector<float2>& tab) {
   tab.assign(twiddle_len(n, D) > 0 ? twiddle_len(n, D) : 1, make_float2(1.f, 0.f));
   const Sched s = sched_for(n);
@@ -350,7 +350,7 @@ bool host_twiddles(int n, int D, std::vector<float2>& tab) {
       for (int j = 0; j < NS; j++) {
         const long m = ((long)r * j) % ((long)NS * R);
         const double ang = 2.0 * M_PI * (double)m / (double)(NS * R);
-        const size_t idx = (size_t)off + (size_t)(r - 1) * NS + j;
+        const size_t idx = (size_t)off + tw_entry(NS, r, j);
         if (idx >= tab.size()) return false;
         tab[idx] = make_float2((float)std::cos(ang), (float)(D * std::sin(ang)));
       }
@@ -2268,7 +2268,7 @@ size_t pwf_plan_describe(const pwf_plan* p, char* buf, size_t len) {
     if (w > 0) o = std::min(sizeof(tmp) - 1, o + (size_t)w);
   };
   auto shape = [&](const ColVariant& v) {
-    put("C%d%s", v.C, v.pipe == MODE_PAIR ? "x2" : v.pipe == 5 ? "tma2" : v.pipe == 4 ? "s2" : v.pipe == 3 ? "p2"
+    put("C%d%s", v.C, v.pipe == MODE_PAIR ? "x2" : v.pipe == 7 ? "s" : v.pipe == 5 ? "tma2" : v.pipe == 4 ? "s2" : v.pipe == 3 ? "p2"
                       : v.pipe == 2 ? "t" : v.pipe ? "p" : "");
     if (v.sched == 1)  // built with the alternative radix schedule: its radices
       for (int i = 0; i < p->kcol->sched_stages[1]; i++) put("%s%d", i ? "." : "@", p->kcol->sched_radix[1][i]);

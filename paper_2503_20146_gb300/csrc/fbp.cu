@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(row_threads(L))
   const bool valid = row < nrows;
   if (!valid) row = nrows - 1;
   const float2* src = in + (size_t)row * nx;
-  const RowLayout<TPF, ROWS * TPF> sm{smem + rr * row_smem_len(L), 1 + rr};
+  const RowLayout<L, ROWS * TPF> sm{smem + rr * row_smem_len(L), 1 + rr};
   float2 v[EPT];
 #pragma unroll
   for (int j = 0; j < EPT; j++) {

@@ -42,15 +42,68 @@ inline namespace PWF_KNS {
 // ---------------------------------------------------------------------------
 // complex helpers
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
-__device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
+// Two-wide FP32 instructions on a register pair (one issue slot for both
+// halves; each half rounds as the scalar instruction does). Reversing the
+// halves of an operand, negating it and using one register for both halves
+// cost no instruction of their own.
+__device__ __forceinline__ uint64_t f2_bits(float2 a) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y));
+  return r;
+}
+__device__ __forceinline__ float2 f2_of(uint64_t a) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
+  return r;
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(f2_bits(a)), "l"(f2_bits(b)));
+  return f2_of(r);
+}
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
+  uint64_t r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(f2_bits(a)), "l"(f2_bits(b)));
+  return f2_of(r);
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(f2_bits(a)), "l"(f2_bits(b)));
+  return f2_of(r);
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(f2_bits(a)), "l"(f2_bits(b)), "l"(f2_bits(c)));
+  return f2_of(r);
+}
+__device__ __forceinline__ float2 swap2(float2 a) { return make_float2(a.y, a.x); }
+
+// Complex arithmetic in two-wide (PK) or scalar instructions.
+template <bool PK = true>
+__device__ __forceinline__ float2 cadd(float2 a, float2 b) {
+  if constexpr (PK) return add2(a, b);
+  else return make_float2(a.x + b.x, a.y + b.y);
+}
+template <bool PK = true>
+__device__ __forceinline__ float2 csub(float2 a, float2 b) {
+  if constexpr (PK) return sub2(a, b);
+  else return make_float2(a.x - b.x, a.y - b.y);
+}
+template <bool PK = true>
+__device__ __forceinline__ float2 cscale(float2 a, float s) {
+  if constexpr (PK) return mul2(a, make_float2(s, s));
+  else return make_float2(a.x * s, a.y * s);
+}
+template <bool PK = true>
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
-  return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
+  if constexpr (PK) return fma2(a, make_float2(b.x, b.x), mul2(swap2(a), make_float2(-b.y, b.y)));
+  else return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
 // a * conj(b)
+template <bool PK = true>
 __device__ __forceinline__ float2 cmulc(float2 a, float2 b) {
-  return make_float2(fmaf(a.x, b.x, a.y * b.y), fmaf(a.y, b.x, -a.x * b.y));
+  if constexpr (PK) return fma2(a, make_float2(b.x, b.x), mul2(swap2(a), make_float2(b.y, -b.y)));
+  else return make_float2(fmaf(a.x, b.x, a.y * b.y), fmaf(a.y, b.x, -a.x * b.y));
 }
 __device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
 __device__ __forceinline__ float cabs2(float2 a) { return fmaf(a.x, a.x, a.y * a.y); }
@@ -63,6 +116,13 @@ template <int DIR>
 __device__ __forceinline__ float2 mul_si(float2 a) {
   if constexpr (DIR == FWD) return make_float2(a.y, -a.x);   // -i a
   else return make_float2(-a.y, a.x);                        // +i a
+}
+
+// a + (s i) b, s = DIR (the products with +-1 of the two-wide form are exact)
+template <bool PK, int DIR>
+__device__ __forceinline__ float2 cadd_i(float2 a, float2 b) {
+  if constexpr (PK) return fma2(swap2(b), DIR == FWD ? make_float2(1.f, -1.f) : make_float2(-1.f, 1.f), a);
+  else return cadd<false>(a, mul_si<DIR>(b));
 }
 
 // exp(s 2 pi i m / 16) for the compile-time exponent m
@@ -81,108 +141,108 @@ __device__ __forceinline__ float2 w16() {
   return make_float2(C[m], DIR == FWD ? -S[m] : S[m]);
 }
 
-template <int DIR, int M>
+template <bool PK, int DIR, int M>
 __device__ __forceinline__ float2 twm16(float2 a) {
   constexpr int m = M & 15;
   if constexpr (m == 0) return a;
   else if constexpr (m == 4) return mul_si<DIR>(a);
   else if constexpr (m == 8) return make_float2(-a.x, -a.y);
   else if constexpr (m == 12) return mul_si<-DIR>(a);
-  else return cmul(a, w16<DIR, m>());
+  else return cmul<PK>(a, w16<DIR, m>());
 }
 
 // ---------------------------------------------------------------------------
 // radix butterflies (in place on x[0..R))
 // ---------------------------------------------------------------------------
-template <int DIR>
+template <bool PK, int DIR>
 __device__ __forceinline__ void dft2(float2* x) {
   float2 a = x[0], b = x[1];
-  x[0] = cadd(a, b);
-  x[1] = csub(a, b);
+  x[0] = cadd<PK>(a, b);
+  x[1] = csub<PK>(a, b);
 }
 
-template <int DIR>
+template <bool PK, int DIR>
 __device__ __forceinline__ void dft3(float2* x) {
   constexpr float H = 0.86602540378443865f;  // sqrt(3)/2
-  float2 s = cadd(x[1], x[2]);
-  float2 d = csub(x[1], x[2]);
+  float2 s = cadd<PK>(x[1], x[2]);
+  float2 d = csub<PK>(x[1], x[2]);
   float2 m = make_float2(fmaf(-0.5f, s.x, x[0].x), fmaf(-0.5f, s.y, x[0].y));
-  float2 r = mul_si<DIR>(cscale(d, H));
-  x[0] = cadd(x[0], s);
-  x[1] = cadd(m, r);
-  x[2] = csub(m, r);
+  float2 r = cscale<PK>(d, H);
+  x[0] = cadd<PK>(x[0], s);
+  x[1] = cadd_i<PK, DIR>(m, r);
+  x[2] = cadd_i<PK, -DIR>(m, r);
 }
 
 // 4-point DFT on elements x[0], x[S], x[2S], x[3S]
-template <int DIR, int S = 1>
+template <bool PK, int DIR, int S = 1>
 __device__ __forceinline__ void dft4s(float2* x) {
-  float2 t0 = cadd(x[0], x[2 * S]);
-  float2 t1 = csub(x[0], x[2 * S]);
-  float2 t2 = cadd(x[S], x[3 * S]);
-  float2 t3 = mul_si<DIR>(csub(x[S], x[3 * S]));
-  x[0] = cadd(t0, t2);
-  x[2 * S] = csub(t0, t2);
-  x[S] = cadd(t1, t3);
-  x[3 * S] = csub(t1, t3);
+  float2 t0 = cadd<PK>(x[0], x[2 * S]);
+  float2 t1 = csub<PK>(x[0], x[2 * S]);
+  float2 t2 = cadd<PK>(x[S], x[3 * S]);
+  float2 t3 = csub<PK>(x[S], x[3 * S]);
+  x[0] = cadd<PK>(t0, t2);
+  x[2 * S] = csub<PK>(t0, t2);
+  x[S] = cadd_i<PK, DIR>(t1, t3);
+  x[3 * S] = cadd_i<PK, -DIR>(t1, t3);
 }
 
-template <int DIR>
-__device__ __forceinline__ void dft4(float2* x) { dft4s<DIR, 1>(x); }
+template <bool PK, int DIR>
+__device__ __forceinline__ void dft4(float2* x) { dft4s<PK, DIR, 1>(x); }
 
 // 8-point: radix-2 split into even/odd 4-point DFTs.
-template <int DIR>
+template <bool PK, int DIR>
 __device__ __forceinline__ void dft8(float2* x) {
   float2 e[4] = {x[0], x[2], x[4], x[6]};
   float2 o[4] = {x[1], x[3], x[5], x[7]};
-  dft4<DIR>(e);
-  dft4<DIR>(o);
-  o[1] = twm16<DIR, 2>(o[1]);
-  o[2] = twm16<DIR, 4>(o[2]);
-  o[3] = twm16<DIR, 6>(o[3]);
+  dft4<PK, DIR>(e);
+  dft4<PK, DIR>(o);
+  o[1] = twm16<PK, DIR, 2>(o[1]);
+  o[2] = twm16<PK, DIR, 4>(o[2]);
+  o[3] = twm16<PK, DIR, 6>(o[3]);
 #pragma unroll
   for (int k = 0; k < 4; k++) {
-    x[k] = cadd(e[k], o[k]);
-    x[k + 4] = csub(e[k], o[k]);
+    x[k] = cadd<PK>(e[k], o[k]);
+    x[k + 4] = csub<PK>(e[k], o[k]);
   }
 }
 
 // 16-point: 4 x 4. Inner 4-point DFTs over j = q + 4m (stride 4), twiddle
 // W16^(q k1), outer 4-point DFTs over q; output index k1 + 4 k2.
-template <int DIR>
+template <bool PK, int DIR>
 __device__ __forceinline__ void dft16(float2* x) {
   float2 y[16];
 #pragma unroll
   for (int q = 0; q < 4; q++) {
     float2 a[4] = {x[q], x[q + 4], x[q + 8], x[q + 12]};
-    dft4<DIR>(a);
+    dft4<PK, DIR>(a);
 #pragma unroll
     for (int k1 = 0; k1 < 4; k1++) y[q * 4 + k1] = a[k1];
   }
   // y[q*4 + k1] *= W16^(q k1)
-  y[1 * 4 + 1] = twm16<DIR, 1>(y[5]);
-  y[1 * 4 + 2] = twm16<DIR, 2>(y[6]);
-  y[1 * 4 + 3] = twm16<DIR, 3>(y[7]);
-  y[2 * 4 + 1] = twm16<DIR, 2>(y[9]);
-  y[2 * 4 + 2] = twm16<DIR, 4>(y[10]);
-  y[2 * 4 + 3] = twm16<DIR, 6>(y[11]);
-  y[3 * 4 + 1] = twm16<DIR, 3>(y[13]);
-  y[3 * 4 + 2] = twm16<DIR, 6>(y[14]);
-  y[3 * 4 + 3] = twm16<DIR, 9>(y[15]);
+  y[1 * 4 + 1] = twm16<PK, DIR, 1>(y[5]);
+  y[1 * 4 + 2] = twm16<PK, DIR, 2>(y[6]);
+  y[1 * 4 + 3] = twm16<PK, DIR, 3>(y[7]);
+  y[2 * 4 + 1] = twm16<PK, DIR, 2>(y[9]);
+  y[2 * 4 + 2] = twm16<PK, DIR, 4>(y[10]);
+  y[2 * 4 + 3] = twm16<PK, DIR, 6>(y[11]);
+  y[3 * 4 + 1] = twm16<PK, DIR, 3>(y[13]);
+  y[3 * 4 + 2] = twm16<PK, DIR, 6>(y[14]);
+  y[3 * 4 + 3] = twm16<PK, DIR, 9>(y[15]);
 #pragma unroll
   for (int k1 = 0; k1 < 4; k1++) {
     float2 a[4] = {y[k1], y[4 + k1], y[8 + k1], y[12 + k1]};
-    dft4<DIR>(a);
+    dft4<PK, DIR>(a);
 #pragma unroll
     for (int k2 = 0; k2 < 4; k2++) x[k1 + 4 * k2] = a[k2];
   }
 }
 
 // exp(s 2 pi i m / 32) for the compile-time exponent m
-template <int DIR, int M>
+template <bool PK, int DIR, int M>
 __device__ __forceinline__ float2 twm32(float2 a) {
   constexpr int m = M & 31;
   if constexpr ((m & 1) == 0) {
-    return twm16<DIR, m / 2>(a);
+    return twm16<PK, DIR, m / 2>(a);
   } else {
     // cos and sin of m*pi/16 for odd m
     constexpr double PI = 3.14159265358979323846;
@@ -198,13 +258,13 @@ __device__ __forceinline__ float2 twm32(float2 a) {
     // rotate by q quarter turns
     constexpr float c = q == 0 ? cr : q == 1 ? -sr : q == 2 ? -cr : sr;
     constexpr float sn = q == 0 ? sr : q == 1 ? cr : q == 2 ? -sr : -cr;
-    return cmul(a, make_float2(c, DIR == FWD ? -sn : sn));
+    return cmul<PK>(a, make_float2(c, DIR == FWD ? -sn : sn));
   }
 }
 
 // 32-point: radix-2 split into the 16-point DFTs of the even and odd
 // samples, combined with the twiddles W32^k.
-template <int DIR>
+template <bool PK, int DIR>
 __device__ __forceinline__ void dft32(float2* x) {
   float2 e[16], o[16];
 #pragma unroll
@@ -212,42 +272,42 @@ __device__ __forceinline__ void dft32(float2* x) {
     e[k] = x[2 * k];
     o[k] = x[2 * k + 1];
   }
-  dft16<DIR>(e);
-  dft16<DIR>(o);
+  dft16<PK, DIR>(e);
+  dft16<PK, DIR>(o);
 #pragma unroll
   for (int k = 0; k < 16; k++) {
     float2 w;
     switch (k) {  // resolved at compile time after unrolling
       case 0: w = o[0]; break;
-      case 1: w = twm32<DIR, 1>(o[1]); break;
-      case 2: w = twm32<DIR, 2>(o[2]); break;
-      case 3: w = twm32<DIR, 3>(o[3]); break;
-      case 4: w = twm32<DIR, 4>(o[4]); break;
-      case 5: w = twm32<DIR, 5>(o[5]); break;
-      case 6: w = twm32<DIR, 6>(o[6]); break;
-      case 7: w = twm32<DIR, 7>(o[7]); break;
-      case 8: w = twm32<DIR, 8>(o[8]); break;
-      case 9: w = twm32<DIR, 9>(o[9]); break;
-      case 10: w = twm32<DIR, 10>(o[10]); break;
-      case 11: w = twm32<DIR, 11>(o[11]); break;
-      case 12: w = twm32<DIR, 12>(o[12]); break;
-      case 13: w = twm32<DIR, 13>(o[13]); break;
-      case 14: w = twm32<DIR, 14>(o[14]); break;
-      default: w = twm32<DIR, 15>(o[15]); break;
+      case 1: w = twm32<PK, DIR, 1>(o[1]); break;
+      case 2: w = twm32<PK, DIR, 2>(o[2]); break;
+      case 3: w = twm32<PK, DIR, 3>(o[3]); break;
+      case 4: w = twm32<PK, DIR, 4>(o[4]); break;
+      case 5: w = twm32<PK, DIR, 5>(o[5]); break;
+      case 6: w = twm32<PK, DIR, 6>(o[6]); break;
+      case 7: w = twm32<PK, DIR, 7>(o[7]); break;
+      case 8: w = twm32<PK, DIR, 8>(o[8]); break;
+      case 9: w = twm32<PK, DIR, 9>(o[9]); break;
+      case 10: w = twm32<PK, DIR, 10>(o[10]); break;
+      case 11: w = twm32<PK, DIR, 11>(o[11]); break;
+      case 12: w = twm32<PK, DIR, 12>(o[12]); break;
+      case 13: w = twm32<PK, DIR, 13>(o[13]); break;
+      case 14: w = twm32<PK, DIR, 14>(o[14]); break;
+      default: w = twm32<PK, DIR, 15>(o[15]); break;
     }
-    x[k] = cadd(e[k], w);
-    x[k + 16] = csub(e[k], w);
+    x[k] = cadd<PK>(e[k], w);
+    x[k + 16] = csub<PK>(e[k], w);
   }
 }
 
-template <int R, int DIR>
+template <bool PK, int R, int DIR>
 __device__ __forceinline__ void dft(float2* x) {
-  if constexpr (R == 2) dft2<DIR>(x);
-  else if constexpr (R == 3) dft3<DIR>(x);
-  else if constexpr (R == 4) dft4<DIR>(x);
-  else if constexpr (R == 8) dft8<DIR>(x);
-  else if constexpr (R == 16) dft16<DIR>(x);
-  else if constexpr (R == 32) dft32<DIR>(x);
+  if constexpr (R == 2) dft2<PK, DIR>(x);
+  else if constexpr (R == 3) dft3<PK, DIR>(x);
+  else if constexpr (R == 4) dft4<PK, DIR>(x);
+  else if constexpr (R == 8) dft8<PK, DIR>(x);
+  else if constexpr (R == 16) dft16<PK, DIR>(x);
+  else if constexpr (R == 32) dft32<PK, DIR>(x);
   else static_assert(R == 2, "unsupported radix");
 }
 
@@ -273,13 +333,19 @@ __host__ __device__ constexpr Sched sched_alt(int n) {
     case 256: return {256, 3, 4, 8, 8, 1, 1, 1};
     case 512: return {512, 3, 8, 8, 8, 1, 1, 1};
     case 768: return {768, 5, 4, 4, 4, 4, 3, 1};
-    case 1024: return {1024, 3, 8, 8, 16, 1, 1, 1};
+    case 1024: return {1024, 3, 16, 8, 8, 1, 1, 1};
     case 1536: return {1536, 6, 4, 4, 4, 4, 2, 3};
     case 2048: return {2048, 3, 8, 16, 16, 1, 1, 1};
     default: return {0, 0, 1, 1, 1, 1, 1, 1};
   }
 }
 
+// 1024 runs two radix-32 stages: what bounds its row passes is the shared-memory
+// and L1 pipe (80 % busy with 16.8.8), and one exchange per transform instead
+// of two halves that traffic; 32 values per thread cost occupancy (16 warps
+// per SM instead of 24). On 180 x 1024^2, 16.8.8 -> 32.32 (ms per launch):
+// row_mul_t 0.763 -> 0.631, row_intensity_pk 0.666 -> 0.579, row_mul_v_pk 0.686 ->
+// 0.590, col_q 0.842 -> 0.770.
 __host__ __device__ constexpr Sched sched_default(int n) {
   switch (n) {
     case 16: return {16, 1, 16, 1, 1, 1, 1, 1};
@@ -292,7 +358,7 @@ __host__ __device__ constexpr Sched sched_default(int n) {
     case 384: return {384, 4, 8, 8, 2, 3, 1, 1};
     case 512: return {512, 3, 16, 8, 4, 1, 1, 1};
     case 768: return {768, 4, 8, 8, 4, 3, 1, 1};
-    case 1024: return {1024, 3, 16, 8, 8, 1, 1, 1};
+    case 1024: return {1024, 2, 32, 32, 1, 1, 1, 1};
     case 1536: return {1536, 4, 8, 8, 8, 3, 1, 1};
     case 2048: return {2048, 3, 16, 16, 8, 1, 1, 1};
     default: return {0, 0, 1, 1, 1, 1, 1, 1};
@@ -332,10 +398,16 @@ __host__ __device__ constexpr int stage_ns(int n, int dir, int k) {
   for (int i = 0; i < k; i++) p *= stage_radix(n, dir, i);
   return p;
 }
+// Twiddles W^(r k), r = 1..R-1, k < NS of a radix-R stage after NS points: two
+// consecutive powers side by side (one 16-byte load), the pairs in [pair][k]
+// order, so that the threads of a transform (consecutive k) read consecutive
+// 16-byte words. An even R leaves its last pair half used.
+__host__ __device__ constexpr int tw_size(int R, int ns) { return (R & ~1) * ns; }
+__host__ __device__ constexpr int tw_entry(int ns, int r, int k) { return ((r - 1) / 2 * ns + k) * 2 + ((r - 1) & 1); }
 // twiddle-table offset of stage k (stage 0 needs none)
 __host__ __device__ constexpr int stage_twoff(int n, int dir, int k) {
   int off = 0;
-  for (int i = 1; i < k; i++) off += (stage_radix(n, dir, i) - 1) * stage_ns(n, dir, i);
+  for (int i = 1; i < k; i++) off += tw_size(stage_radix(n, dir, i), stage_ns(n, dir, i));
   return off;
 }
 __host__ __device__ constexpr int twiddle_len(int n, int dir) { return stage_twoff(n, dir, sched_for(n).s); }
@@ -343,20 +415,26 @@ __host__ __device__ constexpr int twiddle_len(int n, int dir) { return stage_two
 // ---------------------------------------------------------------------------
 // shared-memory layouts
 // ---------------------------------------------------------------------------
-// one transform per row; one padding slot per 16 (breaks the stride-R
-// bank pattern of the first stage's writes). The TPF threads of one row are
-// the only ones that touch it, so a stage barrier covers just them: a named
-// barrier (id 1 + row) when they span several warps, a warp barrier when the
-// row fits in one warp (NT = threads of the block).
-template <int TPF, int NT, bool TWS = false>
+// Padding: one empty slot (row) after every 2^pad_shift(n) of a transform's
+// buffer, which breaks the stride-R0 bank pattern of the first stage's writes:
+// 16 for the schedules whose first radix is 16 or less, 32 for radix 32 (16
+// would leave its writes two to a bank).
+__host__ __device__ constexpr int pad_shift(int n) { return sched_for(n).r0 == 32 ? 5 : 4; }
+
+// one transform per row. The TPF threads of one row are the only ones that
+// touch it, so a stage barrier covers just them: a named barrier (id 1 + row)
+// when they span several warps, a warp barrier when the row fits in one warp
+// (NT = threads of the block).
+template <int N, int NT, bool TWS = false>
 struct RowLayout {
   static constexpr bool kTwShared = TWS;  // the twiddle table handed to the transforms is in shared memory
+  static constexpr bool kPacked = true;
   float2* base;
   int bar;
-  __device__ __forceinline__ float2& operator[](int p) const { return base[p + (p >> 4)]; }
+  __device__ __forceinline__ float2& operator[](int p) const { return base[p + (p >> pad_shift(N))]; }
   __device__ __forceinline__ void sync() const {
-    if constexpr (TPF > 32) {
-      asm volatile("bar.sync %0, %1;\n" ::"r"(bar), "n"(TPF) : "memory");
+    if constexpr (tpf_for(N) > 32) {
+      asm volatile("bar.sync %0, %1;\n" ::"r"(bar), "n"(tpf_for(N)) : "memory");
     } else if constexpr (NT >= 32) {
       __syncwarp();
     } else {
@@ -364,35 +442,34 @@ struct RowLayout {
     }
   }
 };
-__host__ __device__ constexpr int row_smem_len(int n) { return n + n / 16; }
+__host__ __device__ constexpr int row_smem_len(int n) { return n + (n >> pad_shift(n)); }
 
 // C transforms interleaved: element p of column c at row(p)*C + c. With 8 (4)
 // columns a row covers half (a quarter) of the banks, and the first stage of a
 // transform writes rows b*R0 + r, which for the consecutive b of a warp all
-// start on the same bank. One empty row after every 16 (row(p) = p + p/16)
-// spreads those rows evenly for R0 = 16 and R0 = 8, while the aligned groups
-// of consecutive rows of every other access stay contiguous.
-__host__ __device__ constexpr int col_pad_rows(int c) { return (c == 8 || c == 4) ? 1 : 0; }
-__host__ __device__ constexpr int col_row(int p, int c) { return col_pad_rows(c) ? p + (p >> 4) : p; }
-__host__ __device__ constexpr int col_tile_rows(int n, int c) { return col_pad_rows(c) ? n + n / 16 : n; }
-template <int C>
+// start on the same bank. The padding rows (pad_shift) spread those rows
+// evenly, while the aligned groups of consecutive rows of every other access
+// stay contiguous.
+__host__ __device__ constexpr bool col_padded(int c) { return c == 8 || c == 4; }
+template <int N>
+__host__ __device__ constexpr int col_row(int p, int c) { return col_padded(c) ? p + (p >> pad_shift(N)) : p; }
+__host__ __device__ constexpr int col_tile_rows(int n, int c) { return col_padded(c) ? n + (n >> pad_shift(n)) : n; }
+// Column transforms in two-wide instructions (fewer issue slots, but the pairs
+// tie registers together) or scalar ones: two-wide where a thread holds 32
+// values (COL_Q as column pairs at 1024, 32.32: 0.764 ms against 0.843 scalar;
+// 16.8.8: 0.855 against 0.815).
+__host__ __device__ constexpr bool col_packed(int n) { return ept_for(n) >= 32; }
+template <int N, int C>
 struct ColLayout {
+  static constexpr bool kPacked = col_packed(N);
   float2* base;  // already offset by c
-  __device__ __forceinline__ float2& operator[](int p) const { return base[col_row(p, C) * C]; }
+  __device__ __forceinline__ float2& operator[](int p) const { return base[col_row<N>(p, C) * C]; }
   __device__ __forceinline__ void sync() const { __syncthreads(); }
 };
 
 // ---------------------------------------------------------------------------
 // Stockham stages
 // ---------------------------------------------------------------------------
-// Twiddle W^(r k) of a radix-R stage (table entry (r - 1) NS + k of the stage
-// at offset OFF). Every entry is read from the table, which holds all R - 1
-// powers rounded once from double precision. Forming the odd powers as
-// products of two power-of-two entries instead saves table reads but doubles
-// their rounding error, and that error is the same in every row and column of
-// a field: on smooth objects it adds up coherently in the lowest spatial
-// frequencies of the modelled intensity. PWF_TWIDDLE_PRODUCTS restores the
-// products (for measurement).
 // layouts that say so take their twiddle table from shared memory (a plain
 // load); every other table is global and read through the read-only path
 template <class L, class = void>
@@ -404,19 +481,28 @@ struct tw_in_smem<L, std::void_t<decltype(L::kTwShared)>> {
   static constexpr bool value = L::kTwShared;
 };
 
+// The powers W^(r k), r = 1..R-1, of a radix-R stage whose table starts at tw
+// (tw_entry). Every power is read from the table, where each was rounded once
+// from double precision: forming the odd powers as products of two entries
+// would save reads but double their rounding error, and that error is the same
+// in every row and column of a field, so that on smooth objects it adds up
+// coherently in the lowest spatial frequencies of the modelled intensity.
 template <int R, bool TWS = false>
-__device__ __forceinline__ float2 twiddle(const float2* __restrict__ tw, int off, int ns, int k, int r,
-                                          const float2 (&w)[R]) {
-#ifdef PWF_TWIDDLE_PRODUCTS
-  if ((r & (r - 1)) != 0 && R != 3) {
-    const int hi = r >= 16 ? 16 : r >= 8 ? 8 : r >= 4 ? 4 : 2;
-    return cmul(w[hi], w[r - hi]);
+__device__ __forceinline__ void twiddles(const float2* __restrict__ tw, int ns, int k, float2 (&w)[R]) {
+  const float4* __restrict__ t4 = reinterpret_cast<const float4*>(tw) + k;
+#pragma unroll
+  for (int p = 0; p < (R - 1) / 2; p++) {
+    float4 q;
+    if constexpr (TWS) q = t4[p * ns];
+    else q = __ldg(&t4[p * ns]);
+    w[2 * p + 1] = make_float2(q.x, q.y);
+    w[2 * p + 2] = make_float2(q.z, q.w);
   }
-#else
-  (void)w;
-#endif
-  if constexpr (TWS) return tw[off + (r - 1) * ns + k];
-  else return __ldg(&tw[off + (r - 1) * ns + k]);
+  if constexpr (R % 2 == 0) {
+    const float2* __restrict__ t2 = reinterpret_cast<const float2*>(t4 + (R / 2 - 1) * ns);
+    if constexpr (TWS) w[R - 1] = *t2;
+    else w[R - 1] = __ldg(t2);
+  }
 }
 
 // Runs stages [K, S) of the length-N transform with direction DIR on the slot
@@ -436,6 +522,7 @@ __device__ __forceinline__ void fft_stages(float2 (&v)[ept_for(N)], const L& sm,
   constexpr int NS = stage_ns(N, DIR, K);
   constexpr int NB = EPT / R;
   constexpr bool LAST = (K + 1 == S.s);
+  constexpr bool PK = L::kPacked;
   static_assert(EPT % R == 0, "radix must divide the per-thread count");
 
   if constexpr (K > 0) {
@@ -451,18 +538,15 @@ __device__ __forceinline__ void fft_stages(float2 (&v)[ept_for(N)], const L& sm,
     for (int i = 0; i < NB; i++) {
       const int b = t + i * TPF;
       const int k = b % NS;
-      // W^(r k) for r = 1..R-1, each read from the table (computed in double
-      // precision, rounded once)
       float2 w[R];
+      twiddles<R, tw_in_smem<L>::value>(tw + OFF, NS, k, w);
 #pragma unroll
-      for (int r = 1; r < R; r++) w[r] = twiddle<R, tw_in_smem<L>::value>(tw, OFF, NS, k, r, w);
-#pragma unroll
-      for (int r = 1; r < R; r++) v[i * R + r] = cmul(v[i * R + r], w[r]);
-      dft<R, DIR>(&v[i * R]);
+      for (int r = 1; r < R; r++) v[i * R + r] = cmul<PK>(v[i * R + r], w[r]);
+      dft<PK, R, DIR>(&v[i * R]);
     }
   } else {
 #pragma unroll
-    for (int i = 0; i < NB; i++) dft<R, DIR>(&v[i * R]);
+    for (int i = 0; i < NB; i++) dft<PK, R, DIR>(&v[i * R]);
   }
 
   if constexpr (!LAST) {
@@ -489,11 +573,11 @@ __device__ __forceinline__ void fft_run(float2 (&v)[ept_for(N)], const L& sm, in
 // Two interleaved columns per thread (columns c and c + 1 of a ColLayout tile,
 // c even): the same stages on two transforms that share every index, twiddle
 // and barrier, with one 16-byte shared access per element pair.
-template <int C>
+template <int N, int C>
 struct ColPairLayout {
   float2* base;  // offset by the even column c
   __device__ __forceinline__ float4& operator[](int p) const {
-    return *reinterpret_cast<float4*>(base + col_row(p, C) * C);
+    return *reinterpret_cast<float4*>(base + col_row<N>(p, C) * C);
   }
   __device__ __forceinline__ void sync() const { __syncthreads(); }
 };
@@ -519,6 +603,7 @@ __device__ __forceinline__ void fft_stages2(float2 (&v)[ept_for(N)], float2 (&u)
   constexpr int NS = stage_ns(N, DIR, K);
   constexpr int NB = EPT / R;
   constexpr bool LAST = (K + 1 == S.s);
+  constexpr bool PK = col_packed(N);
 
   if constexpr (K > 0) {
     constexpr int OFF = stage_twoff(N, DIR, K);
@@ -538,21 +623,20 @@ __device__ __forceinline__ void fft_stages2(float2 (&v)[ept_for(N)], float2 (&u)
       const int b = t + i * TPF;
       const int k = b % NS;
       float2 w[R];
-#pragma unroll
-      for (int r = 1; r < R; r++) w[r] = twiddle<R, tw_in_smem<L>::value>(tw, OFF, NS, k, r, w);
+      twiddles<R, tw_in_smem<L>::value>(tw + OFF, NS, k, w);
 #pragma unroll
       for (int r = 1; r < R; r++) {
-        v[i * R + r] = cmul(v[i * R + r], w[r]);
-        u[i * R + r] = cmul(u[i * R + r], w[r]);
+        v[i * R + r] = cmul<PK>(v[i * R + r], w[r]);
+        u[i * R + r] = cmul<PK>(u[i * R + r], w[r]);
       }
-      dft<R, DIR>(&v[i * R]);
-      dft<R, DIR>(&u[i * R]);
+      dft<PK, R, DIR>(&v[i * R]);
+      dft<PK, R, DIR>(&u[i * R]);
     }
   } else {
 #pragma unroll
     for (int i = 0; i < NB; i++) {
-      dft<R, DIR>(&v[i * R]);
-      dft<R, DIR>(&u[i * R]);
+      dft<PK, R, DIR>(&v[i * R]);
+      dft<PK, R, DIR>(&u[i * R]);
     }
   }
 

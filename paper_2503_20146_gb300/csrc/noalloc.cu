@@ -68,7 +68,7 @@ __device__ double prop_phase_d(double rho2, double lambda, double L) {
 }
 
 // Twiddle entries of one (length, direction): stage k >= 1 of radix R after
-// NS points holds exp(D 2 pi i r j / (NS R)) at (r - 1) NS + j.
+// NS points holds exp(D 2 pi i r j / (NS R)) at tw_entry(NS, r, j).
 __device__ void fill_twiddles(float2* tab, int n, int D, int idx) {
   const Sched s = sched_for(n);
   for (int k = 1; k < s.s; k++) {
@@ -79,7 +79,7 @@ __device__ void fill_twiddles(float2* tab, int n, int D, int idx) {
       const long m = ((long)r * j) % ((long)NS * R);
       double sn, cs;
       sincospi(2.0 * (double)m / (double)(NS * R), &sn, &cs);
-      tab[off + idx] = make_float2((float)cs, (float)(D * sn));
+      tab[off + tw_entry(NS, r, j)] = make_float2((float)cs, (float)(D * sn));
     }
   }
 }

@@ -132,23 +132,53 @@ __device__ __forceinline__ float2 cexpf2(float2 z) {
   return make_float2(m * c, m * s);
 }
 
+// sin and cos to within an ulp without a slow path in the common range: the
+// phase is reduced by multiples of pi/2 (Cody-Waite, C1 + C2 = pi/2 to 2^-48,
+// one FMA each, so that k <= 2^16 turns leave 2^-33), then odd and even
+// polynomials on [-pi/4, pi/4] (minimax fits of (sin r - r)/r^3 and
+// (cos r - 1 + r^2/2)/r^4 in r^2, weighted for relative error: 2^-27.9 and
+// 2^-33). Against the library sincosf this removes the branch to its
+// large-argument code, which kept the loads of a thread's values from being
+// issued together. Phases beyond 65536 rad take the library routine (out of
+// line: inlined at every value it overflows the instruction cache).
+static __device__ __noinline__ float2 sincos_big(float y) {
+  float2 r;
+  sincosf(y, &r.x, &r.y);
+  return r;
+}
+__device__ __forceinline__ void sincos_acc(float y, float& s, float& c) {
+  constexpr float kInvHalfPi = 0.636619772367581343f;
+  constexpr float kC1 = 1.57079637050628662f;        // float(pi/2)
+  constexpr float kC2 = -4.37113882867379289e-08f;   // float(pi/2 - C1)
+  constexpr float kRound = 12582912.0f;              // 1.5 2^23: the low bits hold the integer
+  const float kr = fmaf(y, kInvHalfPi, kRound);
+  const int n = __float_as_int(kr);
+  const float k = kr - kRound;
+  const float r = fmaf(-k, kC2, fmaf(-k, kC1, y));
+  const float z = r * r;
+  const float sp = fmaf(fmaf(-0.00019511452410370111f, z, 0.008332131430506706f), z, -0.16666653752326965f);
+  const float cp = fmaf(fmaf(fmaf(2.4424791263299994e-05f, z, -0.0013887234963476658f), z, 0.04166664555668831f), z, -0.5f);
+  const float sr = fmaf(r * z, sp, r), cr = fmaf(cp, z, 1.0f);
+  const float sq = (n & 1) ? cr : sr, cq = (n & 1) ? sr : cr;
+  s = __int_as_float(__float_as_int(sq) ^ ((n & 2) << 30));
+  c = __int_as_float(__float_as_int(cq) ^ (((n + 1) & 2) << 30));
+  if (!(fabsf(y) <= 65536.0f)) {
+    const float2 b = sincos_big(y);
+    s = b.x;
+    c = b.y;
+  }
+}
+
 // exp(z) to about one ulp, for the object field x = exp(psi) that enters the
-// forward model and the gradient. The phase is reduced to [-pi, pi] by the same
-// two-constant Cody-Waite step as cexpf2 (so that the library sincosf stays on
-// its short-argument path), and the library sincosf and expf give the rest.
-// The hardware approximations of cexpf2 are 2^-21.4 absolute on the phase and
-// a few ulp on the modulus; both errors are smooth functions of psi, so over a
-// smooth object they add up coherently in the lowest spatial frequencies of
-// the modelled intensity, where the preconditioner of Eq. (11) amplifies them
-// by up to N^2. cexpf2 stays where its errors cancel: the correlation sums.
+// forward model and the gradient. The hardware approximations of cexpf2 are
+// 2^-21.4 absolute on the phase and a few ulp on the modulus; both errors are
+// smooth functions of psi, so over a smooth object they add up coherently in
+// the lowest spatial frequencies of the modelled intensity, where the
+// preconditioner of Eq. (11) amplifies them by up to N^2. cexpf2 stays where
+// its errors cancel: the correlation sums.
 __device__ __forceinline__ float2 cexpf_acc(float2 z) {
-  constexpr float kInv2Pi = 0.159154943091895336f;
-  constexpr float kC1 = 6.28318548202514648f;
-  constexpr float kC2 = -1.74845553146951715e-07f;
-  const float k = rintf(z.y * kInv2Pi);
-  const float r = fmaf(-k, kC2, fmaf(-k, kC1, z.y));
   float s, c;
-  sincosf(r, &s, &c);
+  sincos_acc(z.y, s, c);
   const float m = expf(z.x);
   return make_float2(m * c, m * s);
 }
@@ -214,6 +244,13 @@ __device__ __forceinline__ void row_body(const PassArgs& a, long long row, int t
   (void)proj;
   const size_t rb = (size_t)row * N;
   float2 v[EPT];
+  // Steps that read side inputs and store side outputs read BL values of a
+  // side input before they store: a store may alias the next load as far as
+  // the compiler knows, which would leave one load in flight at a time. On 180
+  // x 1024^2 (ms per launch): row_grad_pack 1.78 -> 1.18, row_nesterov_fft 2.04
+  // -> 1.74; on 24 x 1024^2 row_mode_int 0.162 -> 0.094, col_mode_back 0.187 ->
+  // 0.139, row_exp_fft 0.211 -> 0.072 (with sincos_acc).
+  constexpr int BL = EPT % 8 == 0 ? 8 : EPT;
 
   // Pull this row's side inputs into L2 while the first transform runs.
   if (t == 0) {
@@ -275,7 +312,9 @@ __device__ __forceinline__ void row_body(const PassArgs& a, long long row, int t
     fft_run<N, INV>(v, sm, t, a.tw_inv);
   } else if constexpr (OP == ROW_EXP_FFT) {
 #pragma unroll
-    for (int j = 0; j < EPT; j++) v[j] = cexpf_acc(a.psi[rb + slot_index<N, RS>(t, j)]);
+    for (int j = 0; j < EPT; j++) v[j] = a.psi[rb + slot_index<N, RS>(t, j)];
+#pragma unroll
+    for (int j = 0; j < EPT; j++) v[j] = cexpf_acc(v[j]);
   } else if constexpr (OP == ROW_REAL_FFT) {
 #pragma unroll
     for (int j = 0; j < EPT; j++) v[j] = make_float2(a.y[rb + slot_index<N, RS>(t, j)], 0.f);
@@ -372,30 +411,51 @@ __device__ __forceinline__ void row_body(const PassArgs& a, long long row, int t
   } else if constexpr (OP == ROW_GRAD_OUT) {
     const float s = a.div_maxt2 ? a.gscale / *a.maxt2 : a.gscale;
 #pragma unroll
-    for (int j = 0; j < EPT; j++) {
-      const int x = slot_index<N, RS>(t, j);
-      const float2 xx = cexpf_acc(a.psi[rb + x]);
-      a.g_out[rb + x] = cscale(cmulc(v[j], xx), s);
+    for (int j0 = 0; j0 < EPT; j0 += BL) {
+      float2 ps[BL];
+#pragma unroll
+      for (int j = 0; j < BL; j++) ps[j] = a.psi[rb + slot_index<N, RS>(t, j0 + j)];
+#pragma unroll
+      for (int j = 0; j < BL; j++)
+        a.g_out[rb + slot_index<N, RS>(t, j0 + j)] = cscale(cmulc(v[j0 + j], cexpf_acc(ps[j])), s);
     }
   } else if constexpr (OP == ROW_GRAD_PACK) {
     // g = conj(exp psi) g1 / max|t|^2: Re g out, Im g stays in v for the
     // first row FFT; alpha o psi is formed after it from a second read of psi
     const float s = 1.0f / *a.maxt2;
 #pragma unroll
-    for (int j = 0; j < EPT; j++) {
-      const int x = slot_index<N, RS>(t, j);
-      const float2 g = cscale(cmulc(v[j], cexpf_acc(a.psi[rb + x])), s);
-      a.reg[rb + x] = g.x;
-      v[j] = make_float2(g.y, 0.f);
+    for (int j0 = 0; j0 < EPT; j0 += BL) {
+      float2 ps[BL];
+#pragma unroll
+      for (int j = 0; j < BL; j++) ps[j] = a.psi[rb + slot_index<N, RS>(t, j0 + j)];
+#pragma unroll
+      for (int j = 0; j < BL; j++) {
+        const float2 g = cscale(cmulc(v[j0 + j], cexpf_acc(ps[j])), s);
+        a.reg[rb + slot_index<N, RS>(t, j0 + j)] = g.x;
+        v[j0 + j] = make_float2(g.y, 0.f);
+      }
     }
   } else if constexpr (OP == ROW_NESTEROV_FFT || OP == ROW_NESTEROV) {
     const float beta = *a.beta;
+    constexpr int BN = EPT % 4 == 0 ? 4 : EPT;
 #pragma unroll
-    for (int j = 0; j < EPT; j++) {
+    for (int j0 = 0; j0 < EPT; j0 += BN) {
+     float2 ps[BN], ph[BN];
+     float rg[BN];
+#pragma unroll
+     for (int j = 0; j < BN; j++) {
+      const int x = slot_index<N, RS>(t, j0 + j);
+      ps[j] = a.psi[rb + x];
+      ph[j] = a.phi[rb + x];
+      rg[j] = a.reg[rb + x];
+     }
+#pragma unroll
+     for (int jj = 0; jj < BN; jj++) {
+      const int j = j0 + jj;
       const int x = slot_index<N, RS>(t, j);
-      const float2 p = a.psi[rb + x];
-      const float2 fp = a.phi[rb + x];
-      const float gr = a.reg[rb + x];
+      const float2 p = ps[jj];
+      const float2 fp = ph[jj];
+      const float gr = rg[jj];
       // total direction: preconditioned g plus the regularizer term = Re g + z
       const float2 g = make_float2(gr + v[j].x, v[j].y);
       const float2 f = make_float2(fmaf(-a.eta, g.x, p.x), fmaf(-a.eta, g.y, p.y));
@@ -409,25 +469,38 @@ __device__ __forceinline__ void row_body(const PassArgs& a, long long row, int t
       part[2] += cabs2(xn);
       part[3] += cabs2(xo);
       v[j] = xn;
+     }
     }
   } else if constexpr (OP == ROW_GRADT) {
     const float w2 = 2.0f * a.mode_w;
 #pragma unroll
-    for (int j = 0; j < EPT; j++) {
-      const int x = slot_index<N, RS>(t, j);
-      const float2 u = a.u1[rb + x];
-      float2 gt = cscale(cmulc(v[j], u), w2);
-      if (a.accumulate) gt = cadd(gt, a.gt_scratch[rb + x]);
-      a.gt_scratch[rb + x] = gt;
-      v[j] = cmulc(v[j], __ldg(&a.t[(size_t)yrow * N + x]));
+    for (int j0 = 0; j0 < EPT; j0 += BL) {
+      float2 u[BL], g0[BL];
+#pragma unroll
+      for (int j = 0; j < BL; j++) {
+        const int x = slot_index<N, RS>(t, j0 + j);
+        u[j] = a.u1[rb + x];
+        g0[j] = a.accumulate ? a.gt_scratch[rb + x] : make_float2(0.f, 0.f);
+      }
+#pragma unroll
+      for (int j = 0; j < BL; j++) {
+        const int x = slot_index<N, RS>(t, j0 + j);
+        float2 gt = cscale(cmulc(v[j0 + j], u[j]), w2);
+        if (a.accumulate) gt = cadd(gt, g0[j]);
+        a.gt_scratch[rb + x] = gt;
+        v[j0 + j] = cmulc(v[j0 + j], __ldg(&a.t[(size_t)yrow * N + x]));
+      }
     }
   } else if constexpr (OP == ROW_MODE_INT) {
+    float f0[EPT];
+#pragma unroll
+    for (int j = 0; j < EPT; j++) f0[j] = a.accumulate ? a.f_out[rb + slot_index<N, RS>(t, j)] : 0.f;
 #pragma unroll
     for (int j = 0; j < EPT; j++) {
       const int x = slot_index<N, RS>(t, j);
       if (a.v != nullptr) a.v[rb + x] = v[j];
       float fi = a.mode_w * cabs2(v[j]);
-      if (a.accumulate) fi += a.f_out[rb + x];
+      if (a.accumulate) fi += f0[j];
       a.f_out[rb + x] = fi;
     }
   }
@@ -496,7 +569,7 @@ __global__ void __launch_bounds__(row_threads(N), row_min_blocks(N, OP)) row_ker
   const long long row = (long long)blockIdx.x * ROWS + rr + (long long)a.proj0 * a.ny;
   const int proj = (int)(row / a.ny);
   if (skip_proj(a, proj)) return;  // uniform per CTA (ny % ROWS == 0)
-  const RowLayout<TPF, ROWS * TPF> sm{smem + rr * row_smem_len(N), 1 + rr};
+  const RowLayout<N, ROWS * TPF> sm{smem + rr * row_smem_len(N), 1 + rr};
   float part[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
   row_body<N, OP>(a, row, t, sm, part);
 
@@ -539,20 +612,21 @@ __device__ __forceinline__ void col_tile_filter(const PassArgs& a, const L& sm, 
                                                 size_t base, float2 (&v)[ept_for(N)], float2 (&s2)[S2N],
                                                 float (&part)[5]) {
   constexpr int EPT = ept_for(N);
+  constexpr bool PK = L::kPacked;
   constexpr int RK = last_radix<N, FWD>();
   const size_t ld = (size_t)a.nx;
   if constexpr (OP == COL_Q) {
     const float2 qx = __ldg(&a.qx[col]);
 #pragma unroll
     for (int j = 0; j < EPT; j++) {
-      float2 q = cmul(qx, __ldg(&a.qy[slot_index<N, RK>(t, j)]));
+      float2 q = cmul<PK>(qx, __ldg(&a.qy[slot_index<N, RK>(t, j)]));
       if (a.conj_q) q = cconj(q);
-      v[j] = cscale(cmul(v[j], q), a.scale);
+      v[j] = cscale<PK>(cmul<PK>(v[j], q), a.scale);
     }
   } else if constexpr (OP == COL_IOTF) {
     const float ixv = __ldg(&a.ix[col]) * a.scale;
 #pragma unroll
-    for (int j = 0; j < EPT; j++) v[j] = cscale(v[j], ixv * __ldg(&a.iy[slot_index<N, RK>(t, j)]));
+    for (int j = 0; j < EPT; j++) v[j] = cscale<PK>(v[j], ixv * __ldg(&a.iy[slot_index<N, RK>(t, j)]));
   } else if constexpr (OP == COL_RESID_IOTF2) {
     const float ixv = __ldg(&a.ix[col]);
 #pragma unroll
@@ -562,7 +636,7 @@ __device__ __forceinline__ void col_tile_filter(const PassArgs& a, const L& sm, 
       const float2 yh = a.yhat[base + (size_t)ky * ld];
       const float2 r = make_float2(fmaf(w, v[j].x, -yh.x), fmaf(w, v[j].y, -yh.y));
       part[0] = fmaf(r.x, r.x, fmaf(r.y, r.y, part[0]));
-      v[j] = cscale(r, w * a.scale);
+      v[j] = cscale<PK>(r, w * a.scale);
     }
     part[0] *= a.scale;
   } else if constexpr (OP == COL_PRECOND_REG) {
@@ -632,7 +706,7 @@ __global__ void __launch_bounds__(col_threads(N, C), col_min_blocks_op<OP>(col_t
   const int proj = blockIdx.y + a.proj0;
   const int col = blockIdx.x * C + c;
   if (skip_proj(a, proj)) return;
-  const ColLayout<C> sm{smem + c};
+  const ColLayout<N, C> sm{smem + c};
   float part[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
   col_body<N, OP>(a, proj, col, t, sm, part);
   if constexpr (OP == COL_RESID_IOTF2) block_reduce_add<1>(part, a.acc, proj * NACC + ACC_LOSS, smem);
@@ -646,12 +720,24 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int K>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(K) : "memory"); }
 
-// Persistent, double-buffered: the CTA walks tiles blockIdx.x, +gridDim.x, ...
-// The copy of tile k+1 is one cp.async commit group (16-byte chunks); the wait
-// for tile k is cp.async.wait_group 1, which returns once that group landed.
-template <int N, int OP, int C>
+// rows of a tensor-map box over a column of n rows (a box dimension is at most 256)
+__host__ __device__ constexpr int tma_box_rows(int n) { return n < 256 ? n : 256; }
+// L2 prefetch of one box of a 3-D tensor map (a hint: no completion to wait for)
+__device__ __forceinline__ void tma_prefetch_l2_3d(const CUtensorMap* tm, int x, int y, int z) {
+  asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(tm), "r"(x), "r"(y), "r"(z)
+               : "memory");
+}
+
+// Persistent: the CTA walks tiles blockIdx.x, +gridDim.x, ...
+// NBUF = 2: double-buffered. The copy of tile k+1 is one cp.async commit group
+// (16-byte chunks); the wait for tile k is cp.async.wait_group 1, which returns
+// once that group landed.
+// NBUF = 1: one buffer, so that two CTAs fit on an SM and overlap each other's
+// copy; with a.l2pf, thread 0 prefetches the next tile into L2 through a tensor
+// map once the current one has landed.
+template <int N, int OP, int C, int NBUF>
 __global__ void __launch_bounds__(col_threads(N, C), col_min_blocks_op<OP>(col_threads(N, C), ept_for(N)))
-    col_kernel_pipe(const PassArgs a, int nproj) {
+    col_kernel_pipe(const __grid_constant__ PassArgs a, int nproj, const __grid_constant__ CUtensorMap tmap2) {
   pdl_wait();
   constexpr int EPT = ept_for(N);
   constexpr int NT = col_threads(N, C);
@@ -681,21 +767,39 @@ __global__ void __launch_bounds__(col_threads(N, C), col_min_blocks_op<OP>(col_t
     for (int k = 0; k < CHUNKS / NT; k++) {
       const int q = tid + k * NT;  // chunk q: row q / (C/2), column pair q % (C/2)
       const int row = q / (C / 2), pr = q % (C / 2);
-      cp_async16(buf + col_row(row, C) * C + 2 * pr, a.in + b + (size_t)row * ld + 2 * pr);
+      cp_async16(buf + col_row<N>(row, C) * C + 2 * pr, a.in + b + (size_t)row * ld + 2 * pr);
     }
   };
 
   int tile = blockIdx.x;
-  if (tile < ntiles) prefetch(tile, smem);
+  if (NBUF == 2 && tile < ntiles) prefetch(tile, smem);
   cp_async_commit();
   for (int k = 0; tile < ntiles; k++, tile += gridDim.x) {
-    float2* cur = smem + (k & 1) * TILE;
-    float2* nxt = smem + ((k + 1) & 1) * TILE;
+    float2* cur = smem + (NBUF == 2 ? (k & 1) * TILE : 0);
     const int next = tile + gridDim.x;
-    if (next < ntiles) prefetch(next, nxt);
-    cp_async_commit();
-    cp_async_wait<1>();
-    __syncthreads();
+    if constexpr (NBUF == 2) {
+      float2* nxt = smem + ((k + 1) & 1) * TILE;
+      if (next < ntiles) prefetch(next, nxt);
+      cp_async_commit();
+      cp_async_wait<1>();
+      __syncthreads();
+    } else {
+      prefetch(tile, cur);
+      cp_async_commit();
+      cp_async_wait<0>();
+      if (a.l2pf && tid == 0 && next < ntiles) {
+        constexpr int PB = tma_box_rows(N);
+        int np, nc;
+        (void)tile_base(next, np, nc);
+        if (!skip_proj(a, np))
+#pragma unroll
+          for (int k = 0; k < N / PB; k++) {
+            tma_prefetch_l2_3d(&a.tmap, 2 * nc, k * PB, np);
+            if constexpr (OP == COL_PRECOND_REG) tma_prefetch_l2_3d(&tmap2, 2 * nc, k * PB, np);
+          }
+      }
+      __syncthreads();
+    }
 
     int proj, col0;
     const size_t base = tile_base(tile, proj, col0) + c;
@@ -704,7 +808,7 @@ __global__ void __launch_bounds__(col_threads(N, C), col_min_blocks_op<OP>(col_t
       __syncthreads();
       continue;
     }
-    const ColLayout<C> sm{cur + c};
+    const ColLayout<N, C> sm{cur + c};
     float2 v[EPT];
     float2 s2[(OP == COL_PRECOND_REG) ? EPT : 1];
     float part[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
@@ -765,25 +869,26 @@ template <int N, int OP, class P>
 __device__ __forceinline__ void col_pair_filter(const PassArgs& a, int t, int col, size_t base,
                                                 float2 (&v)[ept_for(N)], float2 (&u)[ept_for(N)], float (&part)[5]) {
   constexpr int EPT = ept_for(N);
+  constexpr bool PK = col_packed(N);
   constexpr int RK = last_radix<N, FWD>();
   const size_t ld = (size_t)a.nx;
   if constexpr (OP == COL_Q) {
-    float2 qa = cscale(__ldg(&a.qx[col]), a.scale), qb = cscale(__ldg(&a.qx[col + 1]), a.scale);
+    float2 qa = cscale<PK>(__ldg(&a.qx[col]), a.scale), qb = cscale<PK>(__ldg(&a.qx[col + 1]), a.scale);
     if (a.conj_q) qa = cconj(qa), qb = cconj(qb);
 #pragma unroll
     for (int j = 0; j < EPT; j++) {
       float2 qy = __ldg(&a.qy[slot_index<N, RK>(t, j)]);
       if (a.conj_q) qy = cconj(qy);
-      v[j] = cmul(v[j], cmul(qa, qy));
-      u[j] = cmul(u[j], cmul(qb, qy));
+      v[j] = cmul<PK>(v[j], cmul<PK>(qa, qy));
+      u[j] = cmul<PK>(u[j], cmul<PK>(qb, qy));
     }
   } else if constexpr (OP == COL_IOTF) {
     const float ia = __ldg(&a.ix[col]) * a.scale, ib = __ldg(&a.ix[col + 1]) * a.scale;
 #pragma unroll
     for (int j = 0; j < EPT; j++) {
       const float iy = __ldg(&a.iy[slot_index<N, RK>(t, j)]);
-      v[j] = cscale(v[j], ia * iy);
-      u[j] = cscale(u[j], ib * iy);
+      v[j] = cscale<PK>(v[j], ia * iy);
+      u[j] = cscale<PK>(u[j], ib * iy);
     }
   } else if constexpr (OP == COL_RESID_IOTF2) {
     const float ia = __ldg(&a.ix[col]), ib = __ldg(&a.ix[col + 1]);
@@ -797,19 +902,11 @@ __device__ __forceinline__ void col_pair_filter(const PassArgs& a, int t, int co
       const float2 rb = make_float2(fmaf(wb, u[j].x, -yh.z), fmaf(wb, u[j].y, -yh.w));
       part[0] = fmaf(ra.x, ra.x, fmaf(ra.y, ra.y, part[0]));
       part[0] = fmaf(rb.x, rb.x, fmaf(rb.y, rb.y, part[0]));
-      v[j] = cscale(ra, wa * a.scale);
-      u[j] = cscale(rb, wb * a.scale);
+      v[j] = cscale<PK>(ra, wa * a.scale);
+      u[j] = cscale<PK>(rb, wb * a.scale);
     }
     part[0] *= a.scale;
   }
-}
-
-// rows of a tensor-map box over a column of n rows (a box dimension is at most 256)
-__host__ __device__ constexpr int tma_box_rows(int n) { return n < 256 ? n : 256; }
-// L2 prefetch of one box of a 3-D tensor map (a hint: no completion to wait for)
-__device__ __forceinline__ void tma_prefetch_l2_3d(const CUtensorMap* tm, int x, int y, int z) {
-  asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(tm), "r"(x), "r"(y), "r"(z)
-               : "memory");
 }
 
 // NBUF = 2: tile k + 1 is copied while tile k is transformed (one CTA per SM
@@ -850,7 +947,7 @@ __global__ void __launch_bounds__(col2_threads(N, C), col2_min_blocks(N, C))
     for (int k = 0; k < CHUNKS / NT; k++) {
       const int q = tid + k * NT;  // chunk q: row q / (C/2), column pair q % (C/2)
       const int row = q / (C / 2), pr = q % (C / 2);
-      cp_async16(buf + col_row(row, C) * C + 2 * pr, a.in + b + (size_t)row * ld + 2 * pr);
+      cp_async16(buf + col_row<N>(row, C) * C + 2 * pr, a.in + b + (size_t)row * ld + 2 * pr);
     }
   };
 
@@ -890,7 +987,7 @@ __global__ void __launch_bounds__(col2_threads(N, C), col2_min_blocks(N, C))
       __syncthreads();
       continue;
     }
-    const ColPairLayout<C> sm{cur + 2 * c2};
+    const ColPairLayout<N, C> sm{cur + 2 * c2};
     float2 v[EPT], u[EPT];
     float part[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
 
@@ -909,7 +1006,7 @@ __global__ void __launch_bounds__(col2_threads(N, C), col2_min_blocks(N, C))
         u[j] = make_float2(q.z, q.w);
       }
       fft_run2<N, FWD>(v, u, sm, t, a.tw_fwd);
-      if constexpr (OP != COL_FFT) col_pair_filter<N, OP, ColPairLayout<C>>(a, t, col, base, v, u, part);
+      if constexpr (OP != COL_FFT) col_pair_filter<N, OP, ColPairLayout<N, C>>(a, t, col, base, v, u, part);
     }
     if constexpr (OP == COL_FFT) {
 #pragma unroll
@@ -973,7 +1070,7 @@ __global__ void __launch_bounds__(col2_threads(N, C), col2_min_blocks(N, C)) col
   const int ntiles = nproj * tiles_per_proj;
   const size_t ldp = 2 * (size_t)a.nx;  // packed rows sit on the even rows of the field
   const bool odd = (t & 1) != 0;        // this thread holds the odd rows 2y' + 1
-  const ColPairLayout<C> sm{smem + 2 * c2};
+  const ColPairLayout<N, C> sm{smem + 2 * c2};
 
   for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int proj = a.proj0 + tile / tiles_per_proj;
@@ -985,7 +1082,7 @@ __global__ void __launch_bounds__(col2_threads(N, C), col2_min_blocks(N, C)) col
       const int q = tid + k * NT;
       const int half = q / CHUNKS, qq = q - half * CHUNKS;
       const int row = qq / (C / 2), pr = qq % (C / 2);
-      cp_async16(smem + col_row(half * H + row, C) * C + 2 * pr,
+      cp_async16(smem + col_row<N>(half * H + row, C) * C + 2 * pr,
                  a.in + pbase + (size_t)row * ldp + (half ? hx : 0) + c0 + 2 * pr);
     }
     cp_async_commit();
@@ -1084,7 +1181,7 @@ __global__ void __launch_bounds__(tpf_for(N)) col_kernel_pk_edge(const PassArgs 
   const int hx = a.nx / 2;
   const size_t pbase = (size_t)proj * a.ny * a.nx;
   const size_t ldp = 2 * (size_t)a.nx;
-  const RowLayout<TPF, TPF> sm{smem, 1};
+  const RowLayout<N, TPF> sm{smem, 1};
   float2 v[EPT];
 #pragma unroll
   for (int j = 0; j < EPT; j++) {
@@ -1299,7 +1396,7 @@ __global__ void __launch_bounds__(col_threads(N, C), col_min_blocks(col_threads(
   const int tiles_per_proj = a.nx / C;
   const int ntiles = nproj * tiles_per_proj;
   const size_t ld = (size_t)a.nx;
-  auto at = [](float2* buf, int col, int p) -> float2& { return buf[col * S + p + (p >> 4)]; };
+  auto at = [](float2* buf, int col, int p) -> float2& { return buf[col * S + p + (p >> pad_shift(N))]; };
 
   auto tile_base = [&](int tile, int& proj, int& col0) -> size_t {
     proj = a.proj0 + tile / tiles_per_proj;
@@ -1338,7 +1435,7 @@ __global__ void __launch_bounds__(col_threads(N, C), col_min_blocks(col_threads(
     }
     const int col = col0 + c;
     const size_t base = tb + c;
-    const RowLayout<TPF, NT> sm{cur + c * S, 1 + c};
+    const RowLayout<N, NT> sm{cur + c * S, 1 + c};
     float2 v[EPT];
     float2 s2[1];
     float part[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
@@ -1407,7 +1504,7 @@ __global__ void __launch_bounds__(col_threads(N, C), col_min_blocks(col_threads(
   const int shifted = ((col - a.mode_mx) % a.nx + a.nx) % a.nx;
   const size_t pb = (size_t)proj * a.ny * a.nx;
   const size_t ld = (size_t)a.nx;
-  const ColLayout<C> sm{smem + c};
+  const ColLayout<N, C> sm{smem + c};
   const int my = ((a.mode_my % N) + N) % N;
   float2 v[EPT];
   if constexpr (MOP == CM_FWD) {
@@ -1428,10 +1525,19 @@ __global__ void __launch_bounds__(col_threads(N, C), col_min_blocks(col_threads(
 #pragma unroll
     for (int j = 0; j < EPT; j++) {
       const int ky = slot_index<N, RK>(t, j);
-      float2 r = cmulc(v[j], cmul(qx, __ldg(&a.qy[ky])));
-      const size_t o = pb + shifted + (size_t)wrap_sub(ky, my, N) * ld;
-      if (a.accumulate) r = cadd(r, a.out[o]);
-      a.out[o] = r;
+      v[j] = cmulc(v[j], cmul(qx, __ldg(&a.qy[ky])));
+    }
+    constexpr int BL = EPT % 8 == 0 ? 8 : EPT;  // accumulated values read before any of them is stored
+#pragma unroll
+    for (int j0 = 0; j0 < EPT; j0 += BL) {
+      float2 old[BL];
+#pragma unroll
+      for (int j = 0; j < BL; j++)
+        old[j] = a.accumulate ? a.out[pb + shifted + (size_t)wrap_sub(slot_index<N, RK>(t, j0 + j), my, N) * ld]
+                              : make_float2(0.f, 0.f);
+#pragma unroll
+      for (int j = 0; j < BL; j++)
+        a.out[pb + shifted + (size_t)wrap_sub(slot_index<N, RK>(t, j0 + j), my, N) * ld] = cadd(v[j0 + j], old[j]);
     }
   }
 }
@@ -1446,6 +1552,7 @@ template <int N, int MOP, int C>
 __global__ void __launch_bounds__(col2_threads(N, C), col2_min_blocks(N, C)) col_mode_kernel2(const PassArgs a) {
   pdl_wait();
   constexpr int EPT = ept_for(N);
+  constexpr bool PK = col_packed(N);
   constexpr int RS = first_radix<N, FWD>();
   constexpr int RK = last_radix<N, FWD>();
   extern __shared__ float2 smem[];
@@ -1462,7 +1569,7 @@ __global__ void __launch_bounds__(col2_threads(N, C), col2_min_blocks(N, C)) col
   const int sh1 = sh0 + 1 < a.nx ? sh0 + 1 : 0;
   const size_t pb = (size_t)proj * a.ny * a.nx;
   const size_t ld = (size_t)a.nx;
-  const ColPairLayout<C> sm{smem + 2 * c2};
+  const ColPairLayout<N, C> sm{smem + 2 * c2};
   const int my = ((a.mode_my % N) + N) % N;
   float2 v[EPT], u[EPT];
   if constexpr (MOP == CM_FWD) {
@@ -1473,8 +1580,8 @@ __global__ void __launch_bounds__(col2_threads(N, C), col2_min_blocks(N, C)) col
       const int ky = slot_index<N, RK>(t, j);
       const float2 qy = __ldg(&a.qy[ky]);
       const size_t o = pb + (size_t)wrap_sub(ky, my, N) * ld;
-      v[j] = cmul(a.in[o + sh0], cmul(qa, qy));
-      u[j] = cmul(a.in[o + sh1], cmul(qb, qy));
+      v[j] = cmul<PK>(a.in[o + sh0], cmul<PK>(qa, qy));
+      u[j] = cmul<PK>(a.in[o + sh1], cmul<PK>(qb, qy));
     }
     fft_run2<N, INV>(v, u, sm, t, a.tw_inv);
 #pragma unroll
@@ -1496,14 +1603,24 @@ __global__ void __launch_bounds__(col2_threads(N, C), col2_min_blocks(N, C)) col
     for (int j = 0; j < EPT; j++) {
       const int ky = slot_index<N, RK>(t, j);
       const float2 qy = __ldg(&a.qy[ky]);
-      const float2 r0 = cmulc(v[j], cmul(qa, qy)), r1 = cmulc(u[j], cmul(qb, qy));
-      float4* o = reinterpret_cast<float4*>(a.out + pb + col + (size_t)wrap_sub(ky, my, N) * ld);
-      float4 q = make_float4(r0.x, r0.y, r1.x, r1.y);
-      if (a.accumulate) {
-        const float4 old = *o;
-        q = make_float4(q.x + old.x, q.y + old.y, q.z + old.z, q.w + old.w);
+      v[j] = cmulc<PK>(v[j], cmul<PK>(qa, qy));
+      u[j] = cmulc<PK>(u[j], cmul<PK>(qb, qy));
+    }
+    constexpr int BL = EPT % 8 == 0 ? 8 : EPT;  // accumulated values read before any of them is stored
+#pragma unroll
+    for (int j0 = 0; j0 < EPT; j0 += BL) {
+      float4 old[BL];
+#pragma unroll
+      for (int j = 0; j < BL; j++)
+        old[j] = a.accumulate ? *reinterpret_cast<const float4*>(
+                                    a.out + pb + col + (size_t)wrap_sub(slot_index<N, RK>(t, j0 + j), my, N) * ld)
+                              : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int j = 0; j < BL; j++) {
+        const float2 p = v[j0 + j], q = u[j0 + j];
+        *reinterpret_cast<float4*>(a.out + pb + col + (size_t)wrap_sub(slot_index<N, RK>(t, j0 + j), my, N) * ld) =
+            make_float4(p.x + old[j].x, p.y + old[j].y, q.x + old[j].z, q.y + old[j].w);
       }
-      *o = q;
     }
   }
 }
@@ -1570,13 +1687,14 @@ struct ColShape {
                                                         colt_smem_bytes(N, C));
       resident = r > 0 ? r : 1;
       return e;
-    } else if constexpr (PIPE == 1) {
-      cudaError_t e = cudaFuncSetAttribute(col_kernel_pipe<N, OP, C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)colp_smem_bytes(N, C));
+    } else if constexpr (PIPE == 1 || PIPE == 7) {
+      constexpr int NB = PIPE == 1 ? 2 : 1;
+      constexpr size_t SM = NB * col_smem_bytes(N, C);
+      cudaError_t e =
+          cudaFuncSetAttribute(col_kernel_pipe<N, OP, C, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM);
       if (e != cudaSuccess) return e;
       int r = 0;
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, col_kernel_pipe<N, OP, C>, col_threads(N, C),
-                                                        colp_smem_bytes(N, C));
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, col_kernel_pipe<N, OP, C, NB>, col_threads(N, C), SM);
       resident = r > 0 ? r : 1;
       return e;
     } else {
@@ -1602,13 +1720,20 @@ struct ColShape {
         b.l2pf = encode_field_tmap(&b.tmap, a.in, a.proj0 + nproj, a.ny, a.nx, C) ? 1 : 0;
         return launch_pass(col_kernel_pipe2<N, OP, C, 1>, dim3(grid), dim3(col2_threads(N, C)), col_smem_bytes(N, C), s,
                            a.pdl, b, nproj);
+      } else if constexpr (PIPE == 7) {
+        PassArgs b = a;
+        CUtensorMap m2{};
+        b.l2pf = encode_field_tmap(&b.tmap, a.in, a.proj0 + nproj, a.ny, a.nx, C) ? 1 : 0;
+        if (OP == COL_PRECOND_REG && b.l2pf) b.l2pf = encode_field_tmap(&m2, a.aux_in, a.proj0 + nproj, a.ny, a.nx, C) ? 1 : 0;
+        return launch_pass(col_kernel_pipe<N, OP, C, 1>, dim3(grid), dim3(col_threads(N, C)), col_smem_bytes(N, C), s,
+                           a.pdl, b, nproj, m2);
       }
       else if constexpr (PIPE == 2)
         return launch_pass(col_kernel_t<N, OP, C>, dim3(grid), dim3(col_threads(N, C)), colt_smem_bytes(N, C), s, a.pdl, a,
                            nproj);
       else
-        return launch_pass(col_kernel_pipe<N, OP, C>, dim3(grid), dim3(col_threads(N, C)), colp_smem_bytes(N, C), s, a.pdl,
-                           a, nproj);
+        return launch_pass(col_kernel_pipe<N, OP, C, 2>, dim3(grid), dim3(col_threads(N, C)), colp_smem_bytes(N, C), s,
+                           a.pdl, a, nproj, CUtensorMap{});
     } else {
       dim3 grid((unsigned)(a.nx / C), (unsigned)nproj);
       return launch_pass(col_kernel<N, OP, C>, grid, dim3(col_threads(N, C)), col_smem_bytes(N, C), s, a.pdl, a);
@@ -1770,6 +1895,8 @@ void add_col_op(LengthKernels& k) {
   add_col_variant<N, OP, 4, 4>(k);
   add_col_variant<N, OP, 8, 5>(k);
   add_col_variant<N, OP, 4, 5>(k);
+  add_col_variant<N, OP, 8, 7>(k);
+  add_col_variant<N, OP, 4, 7>(k);
 }
 
 // the radices of this translation unit's schedule of length N into slot `set`
@@ -1796,6 +1923,7 @@ void add_schedule_shapes(LengthKernels& k) {
     add_col_variant<N, OP, 8, 1>(k);
     add_col_variant<N, OP, 16, 0>(k);
     add_col_variant<N, OP, 8, 0>(k);
+    add_col_variant<N, OP, 8, 7>(k);
   };
   op_shapes(std::integral_constant<int, COL_Q>{});
   op_shapes(std::integral_constant<int, COL_IOTF>{});

@@ -129,7 +129,7 @@ __device__ __forceinline__ void persist_rows(const PassArgs& a, int gw, int GW, 
                                              int only) {
   constexpr int TPF = tpf_for(N), RPW = 32 / TPF;
   const int sub = lane / TPF, t = lane - sub * TPF;
-  const RowLayout<TPF, 32, TWS> sm{wsm + sub * row_smem_len(N), 0};
+  const RowLayout<N, 32, TWS> sm{wsm + sub * row_smem_len(N), 0};
   // every projection's rows, or (only >= 0) those of projection `only`
   const long long per = (long long)a.ny / RPW;
   const long long i0 = only < 0 ? 0 : only * per, items = only < 0 ? a.B * per : i0 + per;
@@ -160,7 +160,7 @@ __device__ __forceinline__ void persist_cols(const PassArgs& a, int gw, int GW, 
                                              int only) {
   constexpr int TPF = tpf_for(N), CPW = 32 / TPF;
   const int c = lane % CPW, t = lane / CPW;
-  const RowLayout<TPF, 32, TWS> sm{wsm + c * row_smem_len(N), 0};
+  const RowLayout<N, 32, TWS> sm{wsm + c * row_smem_len(N), 0};
   const long long per = (long long)a.nx / CPW;
   const long long i0 = only < 0 ? 0 : only * per, items = only < 0 ? a.B * per : i0 + per;
   for (long long it = i0 + gw; it < items; it += GW) {
