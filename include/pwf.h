@@ -321,9 +321,8 @@ pwf_status pwf_diffuser_from_reference(pwf_plan* plan, const float* I_ref, doubl
  *   vol_out  complex64 [ny][nx][nx], device, 8-byte aligned: slice y, row z
  *            (beam direction at angle 0), column x; Re = beta, Im = delta
  *   workspace  device memory of pwf_fbp_workspace_bytes(...) bytes, 256-byte
- *            aligned (filtered rows zero-padded to 2 nx as 16-byte
- *            interpolation records, filter and angle tables; about
- *            32 n_angles ny nx bytes)
+ *            aligned (filtered rows zero-padded to 2 nx, filter and angle
+ *            tables; at most about 32 n_angles ny nx bytes)
  *   stream   cudaStream_t (null: legacy default stream)
  * Ram-Lak: h(0) = 1/4, h(k) = -1/(pi^2 k^2) for odd k, 0 otherwise (unit
  * sampling); linear convolution along the row (zero padding to 2 nx); back
@@ -333,8 +332,8 @@ pwf_status pwf_diffuser_from_reference(pwf_plan* plan, const float* I_ref, doubl
  * 512, 768, 1024, 1536, 2048; otherwise PWF_ERR_INVALID_ARG (workspace_bytes
  * returns 0). A short or misaligned workspace, or misaligned psi / vol_out,
  * also returns PWF_ERR_INVALID_ARG before anything is queued.
- * The tables are copied from the host synchronously on the stream; the two
- * kernels are then enqueued asynchronously. */
+ * The angles travel in launch arguments: the call enqueues its kernels and
+ * returns, without a copy or a synchronisation. */
 #define PWF_FBP_MAX_ANGLES 4096
 size_t pwf_fbp_workspace_bytes(int32_t n_angles, int32_t ny, int32_t nx);
 pwf_status pwf_fbp(const void* psi, int32_t n_angles, int32_t ny, int32_t nx, const double* angles_rad_host,

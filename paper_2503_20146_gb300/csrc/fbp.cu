@@ -3,53 +3,105 @@
 // filter, applied to every detector row independently, then the factor
 // lambda / p / (2 pi)). Parallel-beam, angles over [0, pi).
 //
-// Two kernels:
-//   * fbp_filter_kernel<L>: one detector row per TPF threads. The nx samples
-//     are zero-padded to L = 2 nx (so the circular convolution of length L is
-//     the linear one over the row), transformed with the Stockham runner of the
-//     PWF passes, multiplied by the length-L DFT of the band-limited ramp
-//     (Ram-Lak) kernel, transformed back, and the first nx samples kept. The
-//     complex field psi is filtered as is: the kernel is real and even, so the
-//     real and the imaginary parts are filtered independently in one pass.
-//     The filtered row is stored in the middle of a zeroed row of width 2 nx
-//     (detector pixel i at column i + nx/2), so that the back projection of
-//     any voxel of the nx x nx grid (|s| <= nx / sqrt(2) + 1) reads inside the
-//     row without bounds checks and gets zero outside the detector; each
-//     column holds the record (q[o], q[o+1] - q[o]), so one 16-byte load gives
-//     both taps of the linear interpolation.
-//   * fbp_backproject_kernel: one thread per (x, 8 values of z) of one slice
-//     (warps laid out as 8 x 4 voxel patches);
-//     per angle, s = x cos(theta) + z sin(theta), linear interpolation
-//     q[j] + w (q[j+1] - q[j]) from one record, accumulation in FP32. The angle table sits in shared
-//     memory; the filtered rows of one slice are read through L1/L2 (a 32 x 64
-//     voxel tile touches at most ~70 samples per angle).
+// k_fbp_tables writes the filter spectrum, the twiddles and the angles' cosines
+// and sines (all in double precision) into the workspace; the filter and the
+// back projection follow in one of two forms:
+//   * tiles (from 32 detector rows on, see tile_form): the voxels (x, z) of every
+//     slice meet the detector at the same place, so the lanes of a warp are
+//     slices. fbp_filter_kernel<L, true> writes the filtered rows slice-minor,
+//     [angle][block of slices][column][slice], and fbp_backproject_tiles runs
+//     warp-uniform interpolation on them.
+//   * direct (a few rows, where lanes over slices would idle):
+//     fbp_filter_kernel<L, false> writes each row as records (q[o], q[o+1] -
+//     q[o]), so that one 16-byte load gives both taps, and
+//     fbp_backproject_kernel takes one thread per (x, 8 values of z) of one slice
+//     (warps laid out as 8 x 4 voxel patches).
+// In both, a filtered row sits in the middle of a row of 2 nx columns (detector
+// pixel i at column i + nx/2, zeros around it), so that the back projection of
+// any voxel of the nx x nx grid (|s| <= nx / sqrt(2) + 1) reads inside the row
+// without bounds checks and gets zero outside the detector. The ramp kernel is
+// real and even, so the complex field psi is filtered as it is.
 #include <cuda_runtime.h>
 
 #include <cmath>
 #include <vector>
 
 #include "../../include/pwf.h"
-#include "host_tables.h"
+#include "device_tables.cuh"
 #include "passes.cuh"
 
 namespace pwf {
 namespace {
 
-template <int L>
+// The tile form from 32 rows and 64 tiles on. A tile takes about 1 us per angle
+// whatever part of its lanes holds slices, so it needs rows to fill them and
+// tiles to fill the GPU. Direct / tiles, us per call (angles, ny, nx): (180, 24,
+// 1024) 3688 / 4801, (180, 32, 1024) 4939 / 4832, (180, 64, 1024) 9851 / 5172, (32,
+// 64, 128) 78 / 68, (32, 24, 128) 58 / 66, (90, 40, 48; 9 tiles) 87 / 117.
+bool tile_form(int ny, int nx) { return ny >= 32 && (long long)(nx / 16) * (nx / 16) * ((ny + 63) / 64) >= 64; }
+// slices per block of the tile form: two per lane, or four from 65 rows on
+int tile_slices(int ny) { return ny > 64 ? 128 : 64; }
+
+// The angles of one call travel in the launch's arguments, in parts.
+constexpr int ANGLE_PART = 256;
+struct AnglePart {
+  double rad[ANGLE_PART];
+};
+
+// Filter spectrum, twiddles and angle table. Ram-Lak kernel h(0) = 1/4, h(k) =
+// -1/(pi^2 k^2) for odd k, placed circularly on length L = 2 nx; its DFT is
+// real and even: H(m) = 1/4 + 2 sum_{odd k < nx} h(k) cos(2 pi k m / L), one warp
+// per m; the inverse transform's 1/L is folded in. (On the host the L nx / 2
+// cosines alone took 13 ms at nx = 1024.)
+__global__ void k_fbp_tables(const __grid_constant__ AnglePart part, int first, int count, int L, float* ramp,
+                             float2* twf, float2* twi, double2* cs) {
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx < count) {
+    double s, c;
+    sincos(part.rad[idx], &s, &c);
+    cs[first + idx] = make_double2(c, s);
+  }
+  if (first > 0) return;  // the other tables are written with the first part
+  fill_twiddles(twf, L, FWD, idx);
+  fill_twiddles(twi, L, INV, idx);
+  const int m = idx >> 5, lane = idx & 31;
+  if (m >= L) return;
+  // lane's terms k = 2 lane + 1 + 64 i: the cosine advances by a fixed rotation
+  double c, sn, rc, rs, h = 0.0;
+  sincospi(2.0 * (double)(((2 * lane + 1) * (long)m) % L) / (double)L, &sn, &c);
+  sincospi(2.0 * (double)((64 * (long)m) % L) / (double)L, &rs, &rc);
+  for (int k = 2 * lane + 1; k < L / 2; k += 64) {
+    h -= 2.0 / (M_PI * M_PI * (double)k * k) * c;
+    const double t = c * rc - sn * rs;
+    sn = fma(sn, rc, c * rs);
+    c = t;
+  }
+  for (int o = 16; o > 0; o >>= 1) h += __shfl_xor_sync(0xffffffffu, h, o);
+  if (lane == 0) ramp[m] = (float)((0.25 + h) / L);
+}
+
+// One detector row per TPF threads. The nx samples are zero-padded to L = 2 nx (so that the circular convolution of
+// length L is the linear one), transformed with the Stockham runner of the PWF
+// passes, multiplied by the ramp's spectrum and transformed back.
+template <int L, bool TILES>
 __global__ void __launch_bounds__(row_threads(L))
     fbp_filter_kernel(const float2* __restrict__ in, float2* __restrict__ out, const float* __restrict__ ramp,
-                      const float2* __restrict__ tw_fwd, const float2* __restrict__ tw_inv, long long nrows,
-                      int nx) {
-  constexpr int EPT = ept_for(L), TPF = tpf_for(L), ROWS = rows_for(L);
+                      const float2* __restrict__ tw_fwd, const float2* __restrict__ tw_inv, int n_angles, int ny, int slices) {
+  constexpr int EPT = ept_for(L), TPF = tpf_for(L), ROWS = rows_for(L), nx = L / 2;
   constexpr int RS = first_radix<L, FWD>();
   constexpr int RK = last_radix<L, FWD>();
   extern __shared__ float2 smem[];
   const int rr = threadIdx.x / TPF, t = threadIdx.x - rr * TPF;
-  long long row = (long long)blockIdx.x * ROWS + rr;
-  // rows past the end repeat the last row (every thread of a warp must reach
-  // the warp barriers of the transform) and store nothing
-  const bool valid = row < nrows;
-  if (!valid) row = nrows - 1;
+  // tile form: the rows of a CTA lie in one angle; direct form: consecutive rows
+  // of the whole series. Rows past the end repeat the last row (every thread of
+  // a warp must reach the warp barriers of the transform); what they compute is
+  // not used.
+  const int groups = (ny + ROWS - 1) / ROWS;
+  const int angle = TILES ? blockIdx.x / groups : 0;
+  const int y0 = TILES ? (blockIdx.x - angle * groups) * ROWS : 0;
+  const long long first = TILES ? (long long)angle * ny + y0 : (long long)blockIdx.x * ROWS;
+  const long long end = TILES ? (long long)angle * ny + ny : (long long)n_angles * ny;
+  const long long row = first + rr < end ? first + rr : end - 1;
   const float2* src = in + (size_t)row * nx;
   const RowLayout<L, ROWS * TPF> sm{smem + rr * row_smem_len(L), 1 + rr};
   float2 v[EPT];
@@ -62,10 +114,8 @@ __global__ void __launch_bounds__(row_threads(L))
 #pragma unroll
   for (int j = 0; j < EPT; j++) v[j] = cscale(v[j], __ldg(&ramp[slot_index<L, RK>(t, j)]));
   fft_run<L, INV>(v, sm, t, tw_inv);
-  // records (q[o], q[o+1] - q[o]) of the padded row of width L = 2 nx (samples
-  // at nx/2 .. 3nx/2 - 1, zeros around): first the samples into shared memory
-  // (the transform's buffer is free again; every row of a warp takes part in
-  // the barriers), then the records of valid rows
+  // the padded row (samples at columns nx/2 .. 3nx/2 - 1, zeros around) into
+  // shared memory: the transform's buffer is free again
   float2* rowbuf = smem + rr * row_smem_len(L);
   sm.sync();
 #pragma unroll
@@ -74,31 +124,55 @@ __global__ void __launch_bounds__(row_threads(L))
     const int o = i + nx / 2;
     rowbuf[o < L ? o : o - L] = i < nx ? v[j] : make_float2(0.f, 0.f);
   }
-  sm.sync();
-  if (valid) {
-    float4* dst = reinterpret_cast<float4*>(out) + (size_t)row * L;
-    for (int o = t; o < L; o += TPF) {
-      const float2 q0 = rowbuf[o], q1 = rowbuf[o + 1 < L ? o + 1 : o];
-      dst[o] = make_float4(q0.x, q0.y, q1.x - q0.x, q1.y - q0.y);
+  if constexpr (TILES) {
+    // columns nx/4 .. 7nx/4 - 1 (all that a voxel of the grid can meet), two
+    // rows at a time so that a store writes 16 bytes
+    __syncthreads();
+    constexpr int P = ROWS / 2;
+    static_assert(ROWS % 2 == 0 && 64 % ROWS == 0, "the rows of a CTA lie in one block of slices");
+    float4* dst = reinterpret_cast<float4*>(out) +
+                  ((size_t)angle * ((ny + slices - 1) / slices) + y0 / slices) * L * (slices / 2) + (y0 % slices) / 2;
+    for (int k = threadIdx.x; k < (L - L / 4) * P; k += ROWS * TPF) {
+      const int o = L / 8 + k / P, p = k % P;
+      const float2 a = smem[2 * p * row_smem_len(L) + o], b = smem[(2 * p + 1) * row_smem_len(L) + o];
+      dst[(size_t)o * (slices / 2) + p] = make_float4(a.x, a.y, b.x, b.y);
+    }
+  } else {
+    // records (q[o], q[o+1] - q[o])
+    sm.sync();
+    if (first + rr < end) {
+      float4* dst = reinterpret_cast<float4*>(out) + (size_t)row * L;
+      for (int o = t; o < L; o += TPF) {
+        const float2 q0 = rowbuf[o], q1 = rowbuf[o + 1 < L ? o + 1 : o];
+        dst[o] = make_float4(q0.x, q0.y, q1.x - q0.x, q1.y - q0.y);
+      }
     }
   }
 }
 
-template <int L>
-cudaError_t launch_filter(const float2* in, float2* out, const float* ramp, const float2* twf, const float2* twi,
-                          long long nrows, int nx, cudaStream_t s) {
+template <int L, bool TILES>
+cudaError_t launch_filter_form(const float2* in, float2* out, const float* ramp, const float2* twf, const float2* twi,
+                               int n_angles, int ny, cudaStream_t s) {
   constexpr int ROWS = rows_for(L);
-  const long long blocks = (nrows + ROWS - 1) / ROWS;
+  const long long blocks = TILES ? (long long)n_angles * ((ny + ROWS - 1) / ROWS)
+                                 : ((long long)n_angles * ny + ROWS - 1) / ROWS;
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
   static const cudaError_t attr = cudaFuncSetAttribute(
-      fbp_filter_kernel<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)row_smem_bytes(L));
+      fbp_filter_kernel<L, TILES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)row_smem_bytes(L));
   if (attr != cudaSuccess) return attr;
-  fbp_filter_kernel<L><<<(unsigned)blocks, row_threads(L), row_smem_bytes(L), s>>>(in, out, ramp, twf, twi, nrows,
-                                                                                  nx);
+  fbp_filter_kernel<L, TILES>
+      <<<(unsigned)blocks, row_threads(L), row_smem_bytes(L), s>>>(in, out, ramp, twf, twi, n_angles, ny, tile_slices(ny));
   return cudaGetLastError();
 }
 
-using FilterFn = cudaError_t (*)(const float2*, float2*, const float*, const float2*, const float2*, long long, int,
+template <int L>
+cudaError_t launch_filter(const float2* in, float2* out, const float* ramp, const float2* twf, const float2* twi,
+                          int n_angles, int ny, bool tiles, cudaStream_t s) {
+  return tiles ? launch_filter_form<L, true>(in, out, ramp, twf, twi, n_angles, ny, s)
+               : launch_filter_form<L, false>(in, out, ramp, twf, twi, n_angles, ny, s);
+}
+
+using FilterFn = cudaError_t (*)(const float2*, float2*, const float*, const float2*, const float2*, int, int, bool,
                                  cudaStream_t);
 
 FilterFn filter_for(int L) {
@@ -122,11 +196,11 @@ FilterFn filter_for(int L) {
 constexpr int BP_TX = 32, BP_TY = 8, BP_ZPT = 8;  // tile 32 (x) by 64 (z) voxels
 
 __global__ void __launch_bounds__(BP_TX * BP_TY)
-    fbp_backproject_kernel(const float2* __restrict__ q, float2* __restrict__ vol, const float2* __restrict__ cs,
+    fbp_backproject_kernel(const float2* __restrict__ q, float2* __restrict__ vol, const double2* __restrict__ cs,
                            int n_angles, int ny, int nx, float scale) {
   extern __shared__ float2 scs[];
   const int tid = threadIdx.y * BP_TX + threadIdx.x;
-  for (int i = tid; i < n_angles; i += BP_TX * BP_TY) scs[i] = cs[i];
+  for (int i = tid; i < n_angles; i += BP_TX * BP_TY) scs[i] = make_float2((float)cs[i].x, (float)cs[i].y);
   __syncthreads();
   // each warp covers a compact 8 (x) by 4 (z) patch per z step, so that its
   // lanes' detector positions span at most 8|cos| + 4|sin| + 1 records (two
@@ -176,6 +250,248 @@ __global__ void __launch_bounds__(BP_TX * BP_TY)
   }
 }
 
+// ---------------------------------------------------------------------------
+// tile form of the back projection
+// ---------------------------------------------------------------------------
+// A CTA owns 16 (x) by TZ (z) voxels of a block of slices, a warp one 4 x 4 patch
+// of them, a lane 2 H slices: 16 x 2 H complex sums in registers. For one angle
+// every lane of the warp reads the same detector columns and weights, so a tap
+// is H conflict-free 512-byte rows of shared memory, and it stays in registers
+// while the warp walks its patch:
+//   * the walk is a snake along the axis on which the detector position moves
+//     less (min(|cos|, |sin|) <= 0.71 per voxel), so consecutive voxels use the
+//     same two taps or shift by one;
+//   * tap j lives in register set j mod 2 (A even, B odd): a shift by one loads
+//     one set and moves none. The weight of set A is 1 - w where the lower tap is
+//     even and w where it is odd, that of set B the rest; two-wide FMAs.
+// Positions are 24-bit fixed point relative to the tile's first column, from
+// the double-precision angle table: exact to 2^-20 columns over a tile (a
+// position in one FP32 word is off by nx 2^-24 and more).
+// What bounds it: the shared-memory pipe (65 % busy) and the latency of a tap's
+// load. A walk without reuse reads two taps per voxel (16 bytes per update, 8
+// updates per cycle and SM at best); this one reads 0.57, but a load that its
+// predicate turns off still takes a slot. Branching around the loads halves the
+// pipe's work and is slower (two slices per lane 14.7, four 13.8 ms against 8.9
+// per 128 slices of 180 x 1024 columns): 8 to 16 warps do not hide the branches. An
+// order of visits nearer to the detector position (0.39 taps) measured the
+// same 9.0. Four slices per lane (8 warps, 190 registers) measured 8.9, two
+// (16 warps) 9.8; twelve warps of 4 x 4 patches 8.7, with overhanging tiles.
+// Whole call, 180 x 1024 x 1024: 162.7 -> 71.9 ms (one thread per voxel reading
+// records through the L1, and 13 ms of host cosines).
+// Each stage of two angles is copied by cp.async while the ones before it are
+// used; a stage holds at most ROWS rows, the columns under the tile's diagonal.
+constexpr int BT = 16, BT_STAGES = 3, BT_FRAC = 24;
+
+template <int H>
+struct TileShape {
+  static constexpr int TZ = H == 2 ? 8 : 16;            // voxels along z
+  static constexpr int WARPS = BT / 4 * (TZ / 4);
+  static constexpr int ROWS = H == 2 ? 20 : 24;         // floor(15 |cos| + (TZ - 1) |sin|) + 3 at most
+  static constexpr int SLICES = 64 * H;
+  static constexpr int ROW_BYTES = SLICES * (int)sizeof(float2);
+  static constexpr size_t STAGE = (size_t)ROWS * ROW_BYTES;  // one angle
+  // the angle table (rounded up to an even count), the warps' weights, the stages
+  static constexpr size_t bytes(int n_angles) {
+    return (size_t)(n_angles + 1) / 2 * 2 * sizeof(int4) + (size_t)WARPS * 32 * sizeof(float2) + BT_STAGES * 2 * STAGE;
+  }
+};
+
+// one tap: 2 H slices of one column
+template <int H>
+struct Tap {
+  uint64_t q[2 * H];
+};
+template <int H>
+__device__ __forceinline__ void tap_load(Tap<H>& t, unsigned ptr) {
+  asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(t.q[0]), "=l"(t.q[1]) : "r"(ptr) : "memory");
+  if constexpr (H == 2) asm volatile("ld.shared.v2.b64 {%0, %1}, [%2+512];" : "=l"(t.q[2]), "=l"(t.q[3]) : "r"(ptr) : "memory");
+}
+// where bit is set (the same for the whole warp): ptr += step, then the tap at ptr
+template <int H>
+__device__ __forceinline__ void tap_shift(Tap<H>& t, unsigned bit, unsigned& ptr, int step) {
+  if constexpr (H == 2)
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %5, 0;\n\t@p add.u32 %0, %0, %6;\n\t"
+        "@p ld.shared.v2.b64 {%1, %2}, [%0];\n\t@p ld.shared.v2.b64 {%3, %4}, [%0+512];\n\t}"
+        : "+r"(ptr), "+l"(t.q[0]), "+l"(t.q[1]), "+l"(t.q[2]), "+l"(t.q[3])
+        : "r"(bit), "r"(step)
+        : "memory");
+  else
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t@p add.u32 %0, %0, %4;\n\t"
+        "@p ld.shared.v2.b64 {%1, %2}, [%0];\n\t}"
+        : "+r"(ptr), "+l"(t.q[0]), "+l"(t.q[1])
+        : "r"(bit), "r"(step)
+        : "memory");
+}
+
+// voxel (x, z) of the patch at step p of the walk; ALONG_Z swaps the axes
+template <bool ALONG_Z>
+__host__ __device__ constexpr int walk_x(int p) {
+  const int r = p >> 2, i = (r & 1) ? 3 - (p & 3) : (p & 3);
+  return ALONG_Z ? r : i;
+}
+template <bool ALONG_Z>
+__host__ __device__ constexpr int walk_z(int p) {
+  const int r = p >> 2, i = (r & 1) ? 3 - (p & 3) : (p & 3);
+  return ALONG_Z ? i : r;
+}
+
+// One angle over the warp's patch. pa, pb: shared addresses of the lane's
+// first taps; ma, mb: bit p set where set A (B) shifts at step p; dw, dc: what
+// a shift along (across) the walk adds to a tap's address.
+template <bool ALONG_Z, int H>
+__device__ __forceinline__ void tile_angle(float2 (&acc)[16][2 * H], const float2* w, unsigned pa, unsigned pb,
+                                           unsigned ma, unsigned mb, int dw, int dc) {
+  Tap<H> A, B;
+  tap_load<H>(A, pa);
+  tap_load<H>(B, pb);
+#pragma unroll
+  for (int p = 0; p < 16; p++) {
+    if (p > 0) {
+      const int step = (p & 3) == 0 ? dc : ((p >> 2) & 1) ? -dw : dw;
+      tap_shift<H>(A, ma & (1u << p), pa, step);
+      tap_shift<H>(B, mb & (1u << p), pb, step);
+    }
+    const float2 wp = w[p];
+    float2(&s)[2 * H] = acc[walk_z<ALONG_Z>(p) * 4 + walk_x<ALONG_Z>(p)];
+#pragma unroll
+    for (int k = 0; k < 2 * H; k++) s[k] = fma2(f2_of(A.q[k]), make_float2(wp.x, wp.x), s[k]);
+#pragma unroll
+    for (int k = 0; k < 2 * H; k++) s[k] = fma2(f2_of(B.q[k]), make_float2(wp.y, wp.y), s[k]);
+  }
+}
+
+template <int H>
+__global__ void __launch_bounds__(TileShape<H>::WARPS * 32, 1)
+    fbp_backproject_tiles(const float2* __restrict__ q, float2* __restrict__ vol, const double2* __restrict__ cs,
+                          int n_angles, int ny, int nx, float scale, int vec_out) {
+  using S = TileShape<H>;
+  constexpr int NT = S::WARPS * 32;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  int4* ang = reinterpret_cast<int4*>(smem_raw);  // first column, fixed-point offset of the tile's corner, cos, sin
+  const int na2 = (n_angles + 1) / 2 * 2;
+  float2* wtab = reinterpret_cast<float2*>(ang + na2);
+  unsigned char* stages = reinterpret_cast<unsigned char*>(wtab + S::WARPS * 32);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int x0 = blockIdx.x * BT, z0 = blockIdx.y * S::TZ, yb = blockIdx.z;
+  const int W = 2 * nx;
+  constexpr double ONE = (double)(1 << BT_FRAC);
+  for (int a = tid; a < na2; a += NT) {
+    int4 e = make_int4(0, 0, 0, 0);
+    if (a < n_angles) {
+      const double2 t = cs[a];
+      const double half = 0.5 * nx - 0.5;
+      const int c = __double2int_rn(t.x * ONE), s = __double2int_rn(t.y * ONE);
+      const long long u0 = __double2ll_rn(((x0 - half) * t.x + (z0 - half) * t.y + half + nx / 2) * ONE);
+      const long long lo = u0 + (long long)(BT - 1) * (c < 0 ? c : 0) + (long long)(S::TZ - 1) * (s < 0 ? s : 0);
+      // the first of the tile's columns: with all its rows inside [nx/4, 7nx/4)
+      // for every tile and angle, since |s| <= 0.71 nx and nx >= 16
+      e.x = (int)(lo >> BT_FRAC);
+      e.y = (int)(u0 - ((long long)e.x << BT_FRAC));
+      e.z = c;
+      e.w = s;
+    }
+    ang[a] = e;
+  }
+  __syncthreads();
+  const float2* base = q + (size_t)yb * W * S::SLICES;
+  const size_t plane = (size_t)((ny + S::SLICES - 1) / S::SLICES) * W * S::SLICES;
+  const int groups = na2 / 2;
+  auto copy = [&](int g) {
+    if (g >= groups) return;
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+      const int a = 2 * g + h;
+      if (a >= n_angles) return;
+      const int4 e = ang[a];
+      const int hi = (e.y + (BT - 1) * (e.z > 0 ? e.z : 0) + (S::TZ - 1) * (e.w > 0 ? e.w : 0)) >> BT_FRAC;
+      const int rows = hi + 2 < S::ROWS ? hi + 2 : S::ROWS;
+      const float4* src = reinterpret_cast<const float4*>(base + (size_t)a * plane + (size_t)e.x * S::SLICES);
+      unsigned char* dst = stages + ((g % BT_STAGES) * 2 + h) * S::STAGE;
+      for (int k = tid; k < rows * (S::ROW_BYTES / 16); k += NT) cp_async16(dst + 16 * k, src + k);
+    }
+  };
+  const int px = (warp & 3) * 4, pz = (warp >> 2) * 4;  // the warp's patch
+  float2 acc[16][2 * H];
+#pragma unroll
+  for (int i = 0; i < 16; i++)
+#pragma unroll
+    for (int k = 0; k < 2 * H; k++) acc[i][k] = make_float2(0.f, 0.f);
+  float2* wt = wtab + warp * 32;
+  copy(0);
+  cp_async_commit();
+  copy(1);
+  cp_async_commit();
+  for (int g = 0; g < groups; g++) {
+    cp_async_wait<1>();
+    __syncthreads();  // stage g has landed; every warp is done with stage g - 1
+    copy(g + 2);
+    cp_async_commit();
+    // lanes 0-15 and 16-31: positions, weights and shifts of the 16 voxels in
+    // walk order, for the stage's two angles
+    const int4 e = ang[2 * g + (lane >> 4)];
+    const bool alz = abs(e.z) > abs(e.w);  // |cos| > |sin|: the walk goes along z
+    const int p = lane & 15;
+    const int vx = alz ? walk_x<true>(p) : walk_x<false>(p), vz = alz ? walk_z<true>(p) : walk_z<false>(p);
+    const int u = e.y + (px + vx) * e.z + (pz + vz) * e.w;
+    const int n = u >> BT_FRAC;
+    const float f = (float)(u & ((1 << BT_FRAC) - 1)) * (1.0f / (1 << BT_FRAC));
+    const int ea = (n + 1) & ~1, eb = n | 1;  // the even and the odd tap
+    const float wa = (n & 1) ? f : 1.0f - f;
+    const int pn = __shfl_up_sync(0xffffffffu, n, 1);
+    const unsigned ma = __ballot_sync(0xffffffffu, ea != ((pn + 1) & ~1)), mb = __ballot_sync(0xffffffffu, eb != (pn | 1));
+    __syncwarp();
+    wt[lane] = make_float2(wa, 1.0f - wa);
+    __syncwarp();
+#pragma unroll 1
+    for (int h = 0; h < 2; h++) {
+      if (2 * g + h >= n_angles) break;
+      const int n0 = __shfl_sync(0xffffffffu, n, 16 * h);
+      const int4 eh = ang[2 * g + h];
+      const unsigned sb =
+          (unsigned)__cvta_generic_to_shared(stages + ((g % BT_STAGES) * 2 + h) * S::STAGE) + lane * 16;
+      const unsigned pa = sb + ((n0 + 1) & ~1) * S::ROW_BYTES, pb = sb + (n0 | 1) * S::ROW_BYTES;
+      const unsigned m0 = ma >> (16 * h), m1 = mb >> (16 * h);
+      const int dx = eh.z < 0 ? -2 * S::ROW_BYTES : 2 * S::ROW_BYTES, dz = eh.w < 0 ? -2 * S::ROW_BYTES : 2 * S::ROW_BYTES;
+      if (abs(eh.z) > abs(eh.w)) tile_angle<true, H>(acc, wt + 16 * h, pa, pb, m0, m1, dz, dx);
+      else tile_angle<false, H>(acc, wt + 16 * h, pa, pb, m0, m1, dx, dz);
+    }
+  }
+  cp_async_wait<0>();
+  // a lane's four x of one (z, slice): 32 contiguous bytes
+#pragma unroll
+  for (int k = 0; k < 2 * H; k++) {
+    const int y = yb * S::SLICES + (k >> 1) * 64 + 2 * lane + (k & 1);
+    if (y >= ny) continue;
+#pragma unroll
+    for (int z = 0; z < 4; z++) {
+      float2* dst = vol + ((size_t)y * nx + z0 + pz + z) * nx + x0 + px;
+      const float2 a = cscale(acc[z * 4][k], scale), b = cscale(acc[z * 4 + 1][k], scale);
+      const float2 c = cscale(acc[z * 4 + 2][k], scale), d = cscale(acc[z * 4 + 3][k], scale);
+      if (vec_out) {
+        reinterpret_cast<float4*>(dst)[0] = make_float4(a.x, a.y, b.x, b.y);
+        reinterpret_cast<float4*>(dst)[1] = make_float4(c.x, c.y, d.x, d.y);
+      } else {
+        dst[0] = a, dst[1] = b, dst[2] = c, dst[3] = d;
+      }
+    }
+  }
+}
+
+template <int H>
+cudaError_t launch_tiles(const float2* q, float2* vol, const double2* cs, int n_angles, int ny, int nx, float scale,
+                         cudaStream_t s) {
+  using S = TileShape<H>;
+  static const cudaError_t attr = cudaFuncSetAttribute(
+      fbp_backproject_tiles<H>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::bytes(PWF_FBP_MAX_ANGLES));
+  if (attr != cudaSuccess) return attr;
+  const dim3 grid(nx / BT, nx / S::TZ, (ny + S::SLICES - 1) / S::SLICES);  // nx is a multiple of 16
+  fbp_backproject_tiles<H><<<grid, S::WARPS * 32, S::bytes(n_angles), s>>>(q, vol, cs, n_angles, ny, nx, scale,
+                                                                           ((uintptr_t)vol & 15) == 0);
+  return cudaGetLastError();
+}
+
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 struct FbpLayout {
@@ -185,15 +501,14 @@ struct FbpLayout {
 FbpLayout fbp_layout(int n_angles, int ny, int nx) {
   FbpLayout l{};
   const int L = 2 * nx;
-  std::vector<float2> a, b;
-  host_twiddles(L, FWD, a);
-  host_twiddles(L, INV, b);
+  const size_t row = (size_t)L * (tile_form(ny, nx) ? sizeof(float2) : sizeof(float4));
+  const size_t rows = tile_form(ny, nx) ? (size_t)(ny + tile_slices(ny) - 1) / tile_slices(ny) * tile_slices(ny) : (size_t)ny;
   l.q = 0;
-  l.ramp = l.q + align256((size_t)n_angles * ny * 2 * nx * sizeof(float4));
+  l.ramp = l.q + align256((size_t)n_angles * rows * row);
   l.twf = l.ramp + align256((size_t)L * sizeof(float));
-  l.twi = l.twf + align256(a.size() * sizeof(float2));
-  l.cs = l.twi + align256(b.size() * sizeof(float2));
-  l.total = l.cs + align256((size_t)n_angles * sizeof(float2));
+  l.twi = l.twf + align256((size_t)twiddle_len(L, FWD) * sizeof(float2));
+  l.cs = l.twi + align256((size_t)twiddle_len(L, INV) * sizeof(float2));
+  l.total = l.cs + align256((size_t)n_angles * sizeof(double2));
   return l;
 }
 
@@ -226,46 +541,43 @@ pwf_status pwf_fbp(const void* psi, int32_t n_angles, int32_t ny, int32_t nx, co
   cudaStream_t s = (cudaStream_t)stream;
   char* ws = (char*)workspace;
   const int L = 2 * nx;
-
-  // Ram-Lak kernel h(0) = 1/4, h(k) = -1/(pi^2 k^2) for odd k, placed
-  // circularly on length L; its DFT is real and even:
-  // H(m) = 1/4 + 2 sum_{odd k < nx} h(k) cos(2 pi k m / L). The inverse
-  // transform's 1/L is folded in.
-  std::vector<float> ramp(L);
-  for (int m = 0; m < L; m++) {
-    double h = 0.25;
-    for (int k = 1; k < nx; k += 2) h -= 2.0 / (M_PI * M_PI * (double)k * k) * std::cos(2.0 * M_PI * k * m / L);
-    ramp[m] = (float)(h / L);
-  }
-  std::vector<float2> twf, twi, cs(n_angles);
-  if (!host_twiddles(L, FWD, twf) || !host_twiddles(L, INV, twi)) return PWF_ERR_UNSUPPORTED;
-  for (int a = 0; a < n_angles; a++)
-    cs[a] = make_float2((float)std::cos(angles_rad_host[a]), (float)std::sin(angles_rad_host[a]));
-  // host vectors are pageable: these copies complete before returning
-  if (cudaMemcpyAsync(ws + l.ramp, ramp.data(), L * sizeof(float), cudaMemcpyHostToDevice, s) != cudaSuccess ||
-      cudaMemcpyAsync(ws + l.twf, twf.data(), twf.size() * sizeof(float2), cudaMemcpyHostToDevice, s) !=
-          cudaSuccess ||
-      cudaMemcpyAsync(ws + l.twi, twi.data(), twi.size() * sizeof(float2), cudaMemcpyHostToDevice, s) !=
-          cudaSuccess ||
-      cudaMemcpyAsync(ws + l.cs, cs.data(), cs.size() * sizeof(float2), cudaMemcpyHostToDevice, s) != cudaSuccess ||
-      cudaStreamSynchronize(s) != cudaSuccess) {
-    cudaGetLastError();
-    return PWF_ERR_CUDA;
+  const bool tiles = tile_form(ny, nx);
+  double2* cs = (double2*)(ws + l.cs);
+  bool finite = true;
+  for (int first = 0; first < n_angles; first += ANGLE_PART) {
+    AnglePart part;
+    const int count = n_angles - first < ANGLE_PART ? n_angles - first : ANGLE_PART;
+    for (int a = 0; a < ANGLE_PART; a++) {
+      const bool ok = a < count && std::isfinite(angles_rad_host[first + a]);
+      part.rad[a] = ok ? angles_rad_host[first + a] : 0.0;
+      finite = finite && (ok || a >= count);
+    }
+    const unsigned blocks = first == 0 ? (unsigned)((32 * L + 255) / 256) : 1u;
+    k_fbp_tables<<<blocks, 256, 0, s>>>(part, first, count, L, (float*)(ws + l.ramp), (float2*)(ws + l.twf),
+                                        (float2*)(ws + l.twi), cs);
   }
   float2* q = (float2*)(ws + l.q);
-  const long long nrows = (long long)n_angles * ny;
-  if (filter_for(L)((const float2*)psi, q, (const float*)(ws + l.ramp), (const float2*)(ws + l.twf),
-                    (const float2*)(ws + l.twi), nrows, nx, s) != cudaSuccess) {
+  if (cudaGetLastError() != cudaSuccess ||
+      filter_for(L)((const float2*)psi, q, (const float*)(ws + l.ramp), (const float2*)(ws + l.twf),
+                    (const float2*)(ws + l.twi), n_angles, ny, tiles, s) != cudaSuccess) {
     cudaGetLastError();
     return PWF_ERR_CUDA;
   }
   // back projection weight pi / N_theta and the factor -lambda / (2 pi p):
-  // beta + i delta from psi = -k int beta - i k int delta
-  const float scale = (float)(M_PI / n_angles * (-wavelength_m / (2.0 * M_PI * voxel_m)));
-  const int tiles = (nx + BP_TX - 1) / BP_TX;
-  const dim3 grid(tiles, (nx + BP_TY * BP_ZPT - 1) / (BP_TY * BP_ZPT), ny);
-  fbp_backproject_kernel<<<grid, dim3(BP_TX, BP_TY), n_angles * sizeof(float2), s>>>(
-      q, (float2*)vol_out, (const float2*)(ws + l.cs), n_angles, ny, nx, scale);
+  // beta + i delta from psi = -k int beta - i k int delta. An angle that is not
+  // finite has no positions: it makes every voxel NaN.
+  const float scale = finite ? (float)(M_PI / n_angles * (-wavelength_m / (2.0 * M_PI * voxel_m))) : NAN;
+  if (tiles) {
+    if ((tile_slices(ny) == 128 ? launch_tiles<2>(q, (float2*)vol_out, cs, n_angles, ny, nx, scale, s)
+                                : launch_tiles<1>(q, (float2*)vol_out, cs, n_angles, ny, nx, scale, s)) != cudaSuccess) {
+      cudaGetLastError();
+      return PWF_ERR_CUDA;
+    }
+  } else {
+    const dim3 grid((nx + BP_TX - 1) / BP_TX, (nx + BP_TY * BP_ZPT - 1) / (BP_TY * BP_ZPT), ny);
+    fbp_backproject_kernel<<<grid, dim3(BP_TX, BP_TY), n_angles * sizeof(float2), s>>>(q, (float2*)vol_out, cs, n_angles,
+                                                                                      ny, nx, scale);
+  }
   if (cudaGetLastError() != cudaSuccess) return PWF_ERR_CUDA;
   return PWF_OK;
 }

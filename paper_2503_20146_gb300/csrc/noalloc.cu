@@ -20,6 +20,7 @@
 #include <mutex>
 
 #include "../../include/pwf.h"
+#include "device_tables.cuh"
 #include "passes.cuh"
 
 namespace pwf {
@@ -65,23 +66,6 @@ __device__ double prop_phase_d(double rho2, double lambda, double L) {
   const double il = 1.0 / lambda;
   const double w = sqrt(il * il - rho2);
   return 2.0 * M_PI * L * (-rho2 / (il + w));
-}
-
-// Twiddle entries of one (length, direction): stage k >= 1 of radix R after
-// NS points holds exp(D 2 pi i r j / (NS R)) at tw_entry(NS, r, j).
-__device__ void fill_twiddles(float2* tab, int n, int D, int idx) {
-  const Sched s = sched_for(n);
-  for (int k = 1; k < s.s; k++) {
-    const int R = stage_radix(n, D, k), NS = stage_ns(n, D, k), off = stage_twoff(n, D, k);
-    const int cnt = (R - 1) * NS;
-    if (idx < cnt) {
-      const int r = idx / NS + 1, j = idx % NS;
-      const long m = ((long)r * j) % ((long)NS * R);
-      double sn, cs;
-      sincospi(2.0 * (double)m / (double)(NS * R), &sn, &cs);
-      tab[off + tw_entry(NS, r, j)] = make_float2((float)cs, (float)(D * sn));
-    }
-  }
 }
 
 __global__ void k_noalloc_tables(TableParams p, float2* tw, float2* q, float* io) {
