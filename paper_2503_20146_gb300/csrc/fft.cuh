@@ -262,6 +262,58 @@ __device__ __forceinline__ float2 twm32(float2 a) {
   }
 }
 
+// exp(s 2 pi i m / 24) for the compile-time exponent m
+template <bool PK, int DIR, int M>
+__device__ __forceinline__ float2 twm24(float2 a) {
+  constexpr int m = M % 24;
+  if constexpr (m == 0) return a;
+  else if constexpr (m == 6) return mul_si<DIR>(a);
+  else if constexpr (m == 12) return make_float2(-a.x, -a.y);
+  else if constexpr (m == 18) return mul_si<-DIR>(a);
+  else {
+    // cos of k pi/12, k = 0..6; the angle m pi/12 is q quarter turns and r twelfths of pi
+    constexpr float C[7] = {1.0f, 0.96592582628906829f, 0.86602540378443865f, 0.70710678118654752f,
+                            0.5f, 0.25881904510252076f, 0.0f};
+    constexpr int q = m / 6, r = m % 6;
+    constexpr float cr = C[r], sr = C[6 - r];
+    constexpr float c = q == 0 ? cr : q == 1 ? -sr : q == 2 ? -cr : sr;
+    constexpr float sn = q == 0 ? sr : q == 1 ? cr : q == 2 ? -sr : -cr;
+    return cmul<PK>(a, make_float2(c, DIR == FWD ? -sn : sn));
+  }
+}
+
+// 3 R1-point (R1 = 4 or 8): inner R1-point DFTs over j = q + 3 m, twiddle
+// W_{3 R1}^(q k1), outer 3-point DFTs over q; output index k1 + R1 k2.
+template <bool PK, int R1, int DIR>
+__device__ __forceinline__ void dft3x(float2* x) {
+  constexpr int U = 8 / R1;  // W_{3 R1} = W_24^U
+  float2 y[3][R1];
+#pragma unroll
+  for (int q = 0; q < 3; q++) {
+#pragma unroll
+    for (int m = 0; m < R1; m++) y[q][m] = x[q + 3 * m];
+    if constexpr (R1 == 4) dft4<PK, DIR>(y[q]);
+    else dft8<PK, DIR>(y[q]);
+  }
+#pragma unroll
+  for (int k1 = 0; k1 < R1; k1++) {
+    float2 a[3] = {y[0][k1], y[1][k1], y[2][k1]};
+    switch (k1) {  // resolved at compile time after unrolling
+      case 1: a[1] = twm24<PK, DIR, U>(a[1]); a[2] = twm24<PK, DIR, 2 * U>(a[2]); break;
+      case 2: a[1] = twm24<PK, DIR, 2 * U>(a[1]); a[2] = twm24<PK, DIR, 4 * U>(a[2]); break;
+      case 3: a[1] = twm24<PK, DIR, 3 * U>(a[1]); a[2] = twm24<PK, DIR, 6 * U>(a[2]); break;
+      case 4: a[1] = twm24<PK, DIR, 4 * U>(a[1]); a[2] = twm24<PK, DIR, 8 * U>(a[2]); break;
+      case 5: a[1] = twm24<PK, DIR, 5 * U>(a[1]); a[2] = twm24<PK, DIR, 10 * U>(a[2]); break;
+      case 6: a[1] = twm24<PK, DIR, 6 * U>(a[1]); a[2] = twm24<PK, DIR, 12 * U>(a[2]); break;
+      case 7: a[1] = twm24<PK, DIR, 7 * U>(a[1]); a[2] = twm24<PK, DIR, 14 * U>(a[2]); break;
+      default: break;
+    }
+    dft3<PK, DIR>(a);
+#pragma unroll
+    for (int k2 = 0; k2 < 3; k2++) x[k1 + R1 * k2] = a[k2];
+  }
+}
+
 // 32-point: radix-2 split into the 16-point DFTs of the even and odd
 // samples, combined with the twiddles W32^k.
 template <bool PK, int DIR>
@@ -307,6 +359,8 @@ __device__ __forceinline__ void dft(float2* x) {
   else if constexpr (R == 4) dft4<PK, DIR>(x);
   else if constexpr (R == 8) dft8<PK, DIR>(x);
   else if constexpr (R == 16) dft16<PK, DIR>(x);
+  else if constexpr (R == 12) dft3x<PK, 4, DIR>(x);
+  else if constexpr (R == 24) dft3x<PK, 8, DIR>(x);
   else if constexpr (R == 32) dft32<PK, DIR>(x);
   else static_assert(R == 2, "unsupported radix");
 }
@@ -332,9 +386,9 @@ __host__ __device__ constexpr Sched sched_alt(int n) {
     case 128: return {128, 4, 4, 4, 4, 2, 1, 1};
     case 256: return {256, 3, 4, 8, 8, 1, 1, 1};
     case 512: return {512, 3, 8, 8, 8, 1, 1, 1};
-    case 768: return {768, 5, 4, 4, 4, 4, 3, 1};
+    case 768: return {768, 4, 4, 4, 4, 12, 1, 1};
     case 1024: return {1024, 3, 16, 8, 8, 1, 1, 1};
-    case 1536: return {1536, 6, 4, 4, 4, 4, 2, 3};
+    case 1536: return {1536, 5, 4, 4, 4, 2, 12, 1};
     case 2048: return {2048, 3, 8, 16, 16, 1, 1, 1};
     default: return {0, 0, 1, 1, 1, 1, 1, 1};
   }
@@ -345,21 +399,24 @@ __host__ __device__ constexpr Sched sched_alt(int n) {
 // of two halves that traffic; 32 values per thread cost occupancy (16 warps
 // per SM instead of 24). On 180 x 1024^2, 16.8.8 -> 32.32 (ms per launch):
 // row_mul_t 0.763 -> 0.631, row_intensity_pk 0.666 -> 0.579, row_mul_v_pk 0.686 ->
-// 0.590, col_q 0.842 -> 0.770.
+// 0.590, col_q 0.842 -> 0.770. The multiples of 3 take their factor in one
+// radix-12 or radix-24 stage for the same reason (one exchange less at 24 values
+// per thread): the 25-mode batch of 256^2 .. 2048^2 35.5 -> 32.7 ms, gradients of
+// 9 x 96 x 768 95 -> 86 us. 2048 = 32.64 was slower (64 values per thread spill).
 __host__ __device__ constexpr Sched sched_default(int n) {
   switch (n) {
     case 16: return {16, 1, 16, 1, 1, 1, 1, 1};
     case 32: return {32, 2, 8, 4, 1, 1, 1, 1};
     case 64: return {64, 2, 8, 8, 1, 1, 1, 1};
-    case 96: return {96, 3, 8, 4, 3, 1, 1, 1};
+    case 96: return {96, 2, 8, 12, 1, 1, 1, 1};
     case 128: return {128, 2, 16, 8, 1, 1, 1, 1};
-    case 192: return {192, 3, 8, 8, 3, 1, 1, 1};
+    case 192: return {192, 2, 8, 24, 1, 1, 1, 1};
     case 256: return {256, 2, 16, 16, 1, 1, 1, 1};
-    case 384: return {384, 4, 8, 8, 2, 3, 1, 1};
+    case 384: return {384, 3, 8, 4, 12, 1, 1, 1};
     case 512: return {512, 3, 16, 8, 4, 1, 1, 1};
-    case 768: return {768, 4, 8, 8, 4, 3, 1, 1};
+    case 768: return {768, 3, 8, 8, 12, 1, 1, 1};
     case 1024: return {1024, 2, 32, 32, 1, 1, 1, 1};
-    case 1536: return {1536, 4, 8, 8, 8, 3, 1, 1};
+    case 1536: return {1536, 3, 8, 8, 24, 1, 1, 1};
     case 2048: return {2048, 3, 16, 16, 8, 1, 1, 1};
     default: return {0, 0, 1, 1, 1, 1, 1, 1};
   }
