@@ -89,10 +89,21 @@ __global__ void k_max_abs2(const float2* __restrict__ t, size_t n, float* out) {
   if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<int*>(out), __float_as_int(m));
 }
 
+// The device-side loop of pwf_solve: the last kernel of every iteration sets the
+// while-condition of the graph that holds the iteration. ctl[0] is the
+// iteration limit and ctl[1] the bodies run so far (both written by the host
+// before the launch); the loop ends after ctl[0] bodies whatever the solver
+// state holds, or earlier once the stopping rule has retired every projection.
+__device__ __forceinline__ void loop_control(cudaGraphConditionalHandle h, const DevIter* it, int* ctl, double corr_tol) {
+  const int done = ++ctl[1];
+  const bool more = done < ctl[0] && (corr_tol <= 0.0 || it->n_active > 0);
+  cudaGraphSetConditional(h, more ? 1u : 0u);
+}
 // End of one iteration: per-projection loss / correlation / stopping rule,
-// accumulator reset, and the Nesterov coefficients of the next iteration.
+// accumulator reset, and the Nesterov coefficients of the next iteration; in a
+// graph's loop body (ctl not null) also the loop's condition.
 __global__ void k_finalize(double* acc, int B, int* active, int* iters, double* loss, double* corr,
-                           DevIter* it, double corr_tol) {
+                           DevIter* it, double corr_tol, cudaGraphConditionalHandle h, int* ctl) {
   pdl_wait();
   __shared__ int s_active;
   if (threadIdx.x == 0) s_active = 0;
@@ -106,7 +117,10 @@ __global__ void k_finalize(double* acc, int B, int* active, int* iters, double* 
   atomicAdd(&s_active, na);
   if (nf) it->nonfinite = 1;
   __syncthreads();
-  if (threadIdx.x == 0) finalize_momentum(it, s_active);
+  if (threadIdx.x == 0) {
+    finalize_momentum(it, s_active);
+    if (ctl != nullptr) loop_control(h, it, ctl, corr_tol);
+  }
 }
 
 __global__ void k_state_reset(DevIter* it, int* active, int* iters, double* loss, double* corr, int B) {
@@ -123,20 +137,6 @@ __global__ void k_state_reset(DevIter* it, int* active, int* iters, double* loss
     it->n_active = B;
     it->nonfinite = 0;
     it->status = PWF_OK;
-  }
-}
-
-// The device-side loop of pwf_solve: the last node of every iteration sets the
-// while-condition of the graph that holds the iteration. ctl[0] is the
-// iteration limit and ctl[1] the bodies run so far (both written by the host
-// before the launch); the loop ends after ctl[0] bodies whatever the solver
-// state holds, or earlier once the stopping rule has retired every projection.
-__global__ void k_loop_control(cudaGraphConditionalHandle h, const DevIter* it, int* ctl, double corr_tol) {
-  pdl_wait();
-  if (threadIdx.x == 0) {
-    const int done = ++ctl[1];
-    const bool more = done < ctl[0] && (corr_tol <= 0.0 || it->n_active > 0);
-    cudaGraphSetConditional(h, more ? 1u : 0u);
   }
 }
 
@@ -424,6 +424,8 @@ struct pwf_plan {
   float* maxt2 = nullptr;
   int* kstatus = nullptr;    // set by a kernel whose bounded wait ran out (PWF_ERR_TIMEOUT)
   int* loop_ctl = nullptr;   // device-side loop: {iteration limit, bodies run} (written per solve)
+  cudaGraphConditionalHandle loop_handle = 0;  // while a loop body is captured: its condition,
+  bool in_loop_body = false;                   // set by k_finalize
   size_t ws_bytes = 0;
   std::vector<void*> allocs;
   // solver
@@ -959,7 +961,7 @@ pwf_status fused_iteration(pwf_plan* p, pwf_state* st, const float* y, const flo
     LAUNCH(p, row(p, next_fft ? ROW_NESTEROV_FFT : ROW_NESTEROV, a, nproj_of(p)));
     LAUNCH(p, enqueue(p, "finalize", [&] {
         return launch_pass(k_finalize, dim3(1), dim3(256), 0, p->stream, pdl_of(p), p->acc, a.B, st->active, st->iters,
-                           st->loss, st->corr, st->it, corr_tol);
+                           st->loss, st->corr, st->it, corr_tol, p->loop_handle, p->in_loop_body ? p->loop_ctl : nullptr);
       }));
     return PWF_OK;
   }
@@ -996,7 +998,7 @@ pwf_status fused_iteration(pwf_plan* p, pwf_state* st, const float* y, const flo
   LAUNCH(p, row(p, next_fft ? ROW_NESTEROV_FFT : ROW_NESTEROV, a, nproj_of(p)));
   LAUNCH(p, enqueue(p, "finalize", [&] {
       return launch_pass(k_finalize, dim3(1), dim3(256), 0, p->stream, pdl_of(p), p->acc, a.B, st->active, st->iters,
-                         st->loss, st->corr, st->it, corr_tol);
+                         st->loss, st->corr, st->it, corr_tol, p->loop_handle, p->in_loop_body ? p->loop_ctl : nullptr);
     }));
   if (joint) {
     // joint refinement: step t along the batch sum of g_t (max|t|^2 of the
@@ -1319,8 +1321,8 @@ pwf_status capture_step_graph(pwf_plan* p, F&& body) {
   return PWF_OK;
 }
 
-// The iteration captured into the body of a conditional WHILE node, closed by
-// k_loop_control: one launch runs the loop. PWF_ERR_UNSUPPORTED (with no
+// The iteration captured into the body of a conditional WHILE node, whose
+// condition its k_finalize sets: one launch runs the loop. PWF_ERR_UNSUPPORTED (with no
 // error left pending) when the driver does not take conditional nodes.
 template <class F>
 pwf_status capture_loop_graph(pwf_plan* p, pwf_state* st, double corr_tol, F&& body) {
@@ -1355,13 +1357,10 @@ pwf_status capture_loop_graph(pwf_plan* p, pwf_state* st, double corr_tol, F&& b
     return PWF_ERR_UNSUPPORTED;
   }
   const long long before = p->launches;
+  p->loop_handle = h;
+  p->in_loop_body = true;
   pwf_status r = body();
-  if (r == PWF_OK) {
-    ce = launch_pass(k_loop_control, dim3(1), dim3(32), 0, p->stream, pdl_of(p), h, (const DevIter*)st->it, p->loop_ctl,
-                     corr_tol);
-    if (ce != cudaSuccess) r = cuda_fail(p, ce, "k_loop_control");
-    p->launches++;
-  }
+  p->in_loop_body = false;
   p->graph_kernels = p->launches - before;
   p->launches = before;
   cudaGraph_t captured = nullptr;
@@ -1844,7 +1843,7 @@ pwf_status pwf_step(pwf_plan* p, pwf_state* st, const float* y, const void* t, v
     for (int b = 0; b < p->d.batch; b++)
       if (act[b] && (r = plain_iteration(p, st, y, (const float2*)t, P, b))) return r;
     k_finalize<<<1, 256, 0, p->stream>>>(p->acc, p->d.batch, st->active, st->iters, st->loss, st->corr, st->it,
-                                         corr_tol);
+                                         corr_tol, cudaGraphConditionalHandle{}, nullptr);
     PWF_CUDA(p, cudaGetLastError());
     return PWF_OK;
   }
