@@ -114,10 +114,11 @@ typedef struct pwf_state pwf_state;
                                     output held a NaN or an infinity. Graph
                                     solver only (PWF_ERR_UNSUPPORTED with
                                     PERSISTENT or CLUSTER)                        */
-#define PWF_FLAG_UNPACKED_RESID 0x400u /* the residual passes of the IOTF iteration on
-                                    full complex rows and every column (by default
-                                    the real intensity and residual fields travel
-                                    two rows per complex row, and the column pass
+#define PWF_FLAG_UNPACKED_RESID 0x400u /* the real intensity and residual fields of the
+                                    IOTF form on full complex rows and every column
+                                    (by default they travel two rows per complex
+                                    row, in forward model, gradient and VJP from 2^20
+                                    pixels in the batch on, and the column pass
                                     covers bins kx = 0..nx/2 only, the other half
                                     being their conjugates)                       */
 #define PWF_FLAG_NO_PDL 0x100u   /* launch the passes without programmatic dependent
@@ -372,7 +373,9 @@ size_t pwf_plan_describe(const pwf_plan* plan, char* buf, size_t len);
  * accumulated). Each pass's shapes cover both radix schedules of the length
  * where it has two. pwf_plan_column_shapes returns how many shapes the plan's
  * column length was built with (-1 on a bad argument);
- * pwf_plan_set_column_shape forces one (0-based), replacing the tuned choice. */
+ * pwf_plan_set_column_shape forces one (0-based), replacing the tuned choice
+ * (for pass 6 it also turns the packed forward model, gradient and VJP on for
+ * a plan too small for them). */
 int32_t pwf_plan_column_shapes(const pwf_plan* plan, int32_t pass);
 pwf_status pwf_plan_set_column_shape(pwf_plan* plan, int32_t pass, int32_t shape);
 pwf_status pwf_profile_iteration(pwf_plan* plan, const float* y, const void* t, void* psi, int32_t iters,

@@ -403,6 +403,7 @@ struct pwf_plan {
   const LengthKernels* krow = nullptr;  // length nx
   const LengthKernels* kcol = nullptr;  // length ny
   int colsel[NUM_COL_OPS] = {};  // chosen column-pass shape per op
+  bool pk_asked = false;         // a packed-residual shape was set by the caller
   float coltime[NUM_COL_OPS][MAX_COL_VARIANTS] = {};  // tuning times (ms per launch)
   int modesel[2] = {0, 0};                              // chosen mode column-pass shape (CM_FWD, CM_BACK)
   float modetime[2][MAX_MODE_VARIANTS] = {};            // their tuning times
@@ -696,6 +697,14 @@ cudaError_t row(pwf_plan* p, int op, PassArgs a, int nproj) {
   cudaError_t e = enqueue(p, kRowNames[op], [&] { return p->krow->row[op](a, nproj, p->stream); });
   return e != cudaSuccess ? e : scan_pass(p, kRowNames[op], a, nproj, op, true);
 }
+// packed real row passes
+const char* const kPkRowNames[NUM_PKROW_OPS] = {"row_real_fft_pk", "row_real_out_pk", "row_resid_pk"};
+cudaError_t row_pk(pwf_plan* p, int op, PassArgs a, int nproj) {
+  a = row_args(p, a);
+  cudaError_t e = enqueue(p, kPkRowNames[op], [&] { return p->krow->row_pk[op](a, nproj, p->stream); });
+  if (e == cudaSuccess && op == PKROW_OUT) e = scan_output(p, kPkRowNames[op], a.f_out, a.proj0, nproj, 1);
+  return e;
+}
 // the column-axis twiddles of the radix schedule a column shape was built with
 PassArgs sched_tables(const pwf_plan* p, PassArgs a, int sched) {
   a.tw_fwd = sched == 1 ? p->ay.tw_fwd_alt : p->ay.tw_fwd;
@@ -707,8 +716,13 @@ cudaError_t col(pwf_plan* p, int op, PassArgs a, int nproj) {
   a = sched_tables(p, col_args(p, a), p->kcol->colv[op][p->colsel[op]].sched);
   cudaError_t e =
       enqueue(p, kColNames[op], [&] { return p->kcol->colv[op][p->colsel[op]].launch(a, nproj, p->stream); });
-  if (op == COL_RESID_PK) p->launches++;  // its second kernel: bins 0 and nx/2
   return e != cudaSuccess ? e : scan_pass(p, kColNames[op], a, nproj, op, false);
+}
+// the IOTF filter on packed rows, in the shape chosen for COL_RESID_PK
+cudaError_t col_iotf_pk(pwf_plan* p, PassArgs a, int nproj) {
+  const ColVariant& v = p->kcol->iotf_pk[p->colsel[COL_RESID_PK]];
+  a = sched_tables(p, col_args(p, a), v.sched);
+  return enqueue(p, "col_iotf_pk", [&] { return v.launch(a, nproj, p->stream); });
 }
 cudaError_t col_q(pwf_plan* p, PassArgs a, int which, int conj, int nproj) {
   a = sched_tables(p, colq_args(p, a, which, conj), p->kcol->colv[COL_Q][p->colsel[COL_Q]].sched);
@@ -920,17 +934,28 @@ pwf_status modal_resid(pwf_plan* p, const float* y, const int* active) {
              : cuda_fail(p, cudaGetLastError(), "k_modal_resid");
 }
 
-// The residual passes of the IOTF iteration take the packed form (two real
-// rows per complex row, columns kx and nx - kx from one transform pair) where
-// the column length has packed shapes, unless PWF_FLAG_UNPACKED_RESID.
-bool packed_resid(const pwf_plan* p) {
-  return !(p->d.flags & PWF_FLAG_UNPACKED_RESID) && p->kcol->ncolv[COL_RESID_PK] > 0;
-}
-
 // A packed-residual shape covers C of the nx/2 positions per tile: it fits a
 // plan whose nx/2 it divides. Every other shape fits every plan of its length.
 bool shape_fits(const pwf_plan* p, int op, const ColVariant& v) {
   return op != COL_RESID_PK || (p->d.nx / 2) % v.C == 0;
+}
+
+// The residual passes of the IOTF iteration take the packed form (two real
+// rows per complex row, columns kx and nx - kx from one transform pair) where
+// the column length has a packed shape that fits the plan, unless
+// PWF_FLAG_UNPACKED_RESID.
+bool packed_resid(const pwf_plan* p) {
+  return !(p->d.flags & PWF_FLAG_UNPACKED_RESID) && p->kcol->ncolv[COL_RESID_PK] > 0 &&
+         shape_fits(p, COL_RESID_PK, p->kcol->colv[COL_RESID_PK][p->colsel[COL_RESID_PK]]);
+}
+// The forward model, gradient and VJP carry their real fields (|v|^2, f, the
+// residual, the cotangent) packed too, from 2^20 pixels on (or when a packed
+// shape was asked for): half the column transforms and of the bytes, but
+// longer chains per CTA, which small launches do not hide. Unpacked / packed, us
+// per forward model: 9 x 96 x 768 34 / 39, 512^2 26 / 26, 1024^2 44 / 46, 4 x 512^2 41 /
+// 38, 2048^2 141 / 129; gradient 81 / 91, 68 / 68, 114 / 116, 100 / 93, 321 / 295.
+bool packed_real(const pwf_plan* p) {
+  return packed_resid(p) && (p->pk_asked || (long long)p->d.batch * p->d.ny * p->d.nx >= 1ll << 20);
 }
 
 // one fused iteration (or the body of pwf_step): X must hold F_row{exp psi}
@@ -1469,7 +1494,7 @@ pwf_status pwf_plan_create(const pwf_plan_desc* desc, pwf_plan** out) {
     return PWF_ERR_CUDA;
   }
   for (int op = 0; op < NUM_ROW_OPS; op++)
-    if (p->krow->row_prep[op]() != cudaSuccess) {
+    if (p->krow->row_prep[op]() != cudaSuccess || (op < NUM_PKROW_OPS && p->krow->row_pk_prep[op]() != cudaSuccess)) {
       cudaGetLastError();
       pwf_plan_destroy(p);
       return PWF_ERR_CUDA;
@@ -1483,7 +1508,7 @@ pwf_status pwf_plan_create(const pwf_plan_desc* desc, pwf_plan** out) {
       }
   for (int op = 0; op < NUM_COL_OPS; op++)
     for (int v = 0; v < p->kcol->ncolv[op]; v++)
-      if (p->kcol->colv[op][v].prep() != cudaSuccess) {
+      if (p->kcol->colv[op][v].prep() != cudaSuccess || (op == COL_RESID_PK && p->kcol->iotf_pk[v].prep() != cudaSuccess)) {
         cudaGetLastError();
         pwf_plan_destroy(p);
         return PWF_ERR_CUDA;
@@ -1612,6 +1637,12 @@ pwf_status pwf_forward(pwf_plan* p, const void* psi, const void* t, float* f) {
     LAUNCH(p, row(p, ROW_INTENSITY_OUT, a, a.B));
   } else {
     a.v = nullptr;
+    if (packed_real(p)) {  // |v|^2 and f are real: two rows per complex row, half the columns
+      LAUNCH(p, row(p, ROW_INTENSITY_PK, a, a.B));
+      LAUNCH(p, col_iotf_pk(p, a, a.B));
+      LAUNCH(p, row_pk(p, PKROW_OUT, a, a.B));
+      return PWF_OK;
+    }
     LAUNCH(p, row(p, ROW_INTENSITY, a, a.B));
     LAUNCH(p, col(p, COL_IOTF, a, a.B));
     LAUNCH(p, row(p, ROW_REAL_OUT, a, a.B));
@@ -1654,11 +1685,19 @@ pwf_status pwf_gradient(pwf_plan* p, const void* psi, const void* t, const float
     LAUNCH(p, row(p, ROW_COH_RESID, a, a.B));
   } else {
     a.v = p->V;
-    LAUNCH(p, row(p, ROW_INTENSITY, a, a.B));   // |v|^2, v kept
-    LAUNCH(p, col(p, COL_IOTF, a, a.B));        // f = F^-1{IOTF F{|v|^2}}
-    LAUNCH(p, row(p, ROW_RESID, a, a.B));       // e = y - f; loss; -e
-    LAUNCH(p, col(p, COL_IOTF, a, a.B));        // F^-1{IOTF F{-e}}
-    LAUNCH(p, row(p, ROW_MUL_V, a, a.B));       // v g
+    if (packed_real(p)) {  // the same five steps on real fields packed two rows per complex row
+      LAUNCH(p, row(p, ROW_INTENSITY_PK, a, a.B));
+      LAUNCH(p, col_iotf_pk(p, a, a.B));
+      LAUNCH(p, row_pk(p, PKROW_RESID, a, a.B));
+      LAUNCH(p, col_iotf_pk(p, a, a.B));
+      LAUNCH(p, row(p, ROW_MUL_V_PK, a, a.B));
+    } else {
+      LAUNCH(p, row(p, ROW_INTENSITY, a, a.B));   // |v|^2, v kept
+      LAUNCH(p, col(p, COL_IOTF, a, a.B));        // f = F^-1{IOTF F{|v|^2}}
+      LAUNCH(p, row(p, ROW_RESID, a, a.B));       // e = y - f; loss; -e
+      LAUNCH(p, col(p, COL_IOTF, a, a.B));        // F^-1{IOTF F{-e}}
+      LAUNCH(p, row(p, ROW_MUL_V, a, a.B));       // v g
+    }
   }
   if ((r = fused_backprop(p, a, (const float2*)t, false, a.B))) return r;
   a.psi = P;
@@ -1701,13 +1740,9 @@ pwf_status pwf_forward_vjp(pwf_plan* p, const void* psi, const void* t, const fl
       LAUNCH(p, row(p, ROW_MUL_T, b, a.B));
       b.u1 = nullptr;
       LAUNCH(p, col_q(p, b, 2, 0, a.B));
-      b.out = p->V;
-      LAUNCH(p, row(p, ROW_IFFT, b, a.B));          // v_j
-      b.v = p->V;
-      b.y = grad_f;
       b.out = p->M;
-      LAUNCH(p, row(p, ROW_MODE_VG, b, a.B));       // v_j dL/df
-      b.in = p->M;
+      b.y = grad_f;
+      LAUNCH(p, row(p, ROW_COH_VJP, b, a.B));       // v_j dL/df, v_j in registers only
       LAUNCH(p, col_q(p, b, 2, 1, a.B));            // P2^H
       if (grad_t) {
         b.u1 = p->S;
@@ -1744,6 +1779,19 @@ pwf_status pwf_forward_vjp(pwf_plan* p, const void* psi, const void* t, const fl
   if (p->coherent) {
     a.y = grad_f;
     LAUNCH(p, row(p, ROW_COH_VJP, a, a.B));     // v grad_f
+  } else if (packed_real(p)) {
+    // G = F^-1{IOTF F{grad_f}} on its own (packed rows in V, G in REG), then v G
+    // in the pass that inverts v
+    PassArgs b = a;
+    b.in = p->V;
+    b.out = p->V;
+    b.y = grad_f;
+    b.f_out = p->REG;
+    LAUNCH(p, row_pk(p, PKROW_FFT, b, a.B));
+    LAUNCH(p, col_iotf_pk(p, b, a.B));
+    LAUNCH(p, row_pk(p, PKROW_OUT, b, a.B));
+    a.y = p->REG;
+    LAUNCH(p, row(p, ROW_COH_VJP, a, a.B));     // v G
   } else {
     a.out = p->V;
     LAUNCH(p, row(p, ROW_IFFT, a, a.B));        // v
@@ -2247,7 +2295,8 @@ pwf_status pwf_plan_set_column_shape(pwf_plan* p, int32_t pass, int32_t shape) {
     return fail(p, PWF_ERR_UNSUPPORTED, "column shape does not fit this plan's nx");
   if (pass < NUM_COL_OPS)
     p->colsel[pass] = shape;
-  else
+  if (pass == COL_RESID_PK) p->pk_asked = true;
+  if (pass >= NUM_COL_OPS)
     p->modesel[pass - NUM_COL_OPS] = shape;
   if (p->graph) {  // the captured iteration used the previous shapes
     cudaGraphExecDestroy(p->graph);

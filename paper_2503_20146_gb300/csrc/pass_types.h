@@ -97,6 +97,14 @@ enum RowOp : int {
   NUM_ROW_OPS
 };
 
+// packed real row passes (one transform per pair of rows)
+enum PkRowOp : int {
+  PKROW_FFT = 0,       // two real rows (y) -> FFT -> packed row
+  PKROW_OUT,           // packed row -> IFFT -> two real rows (f_out)
+  PKROW_RESID,         // packed row -> IFFT -> f; e = y - f; loss; -e -> FFT -> packed row
+  NUM_PKROW_OPS
+};
+
 enum ColOp : int {
   COL_Q = 0,           // FFT -> * Q (or conj Q) -> IFFT
   COL_IOTF,            // FFT -> * IOTF -> IFFT
@@ -142,7 +150,10 @@ struct LengthKernels {
   int sched_stages[2];
   PassFn row[NUM_ROW_OPS];
   PrepFn row_prep[NUM_ROW_OPS];
+  PassFn row_pk[NUM_PKROW_OPS];
+  PrepFn row_pk_prep[NUM_PKROW_OPS];
   ColVariant colv[NUM_COL_OPS][MAX_COL_VARIANTS];
+  ColVariant iotf_pk[MAX_COL_VARIANTS];  // the packed IOTF filter in the shapes of colv[COL_RESID_PK]
   int ncolv[NUM_COL_OPS];
   // mode column passes (CM_FWD, CM_BACK): shapes, the default first
   ColVariant colmodev[2][MAX_MODE_VARIANTS];

@@ -582,6 +582,76 @@ __global__ void __launch_bounds__(row_threads(N), row_min_blocks(N, OP)) row_ker
 }
 
 // ---------------------------------------------------------------------------
+// packed real row passes
+// ---------------------------------------------------------------------------
+// Row passes whose fields are real on the real-space side: one transform per
+// packed row y' (rows 2y' and 2y' + 1 of the field as real and imaginary part),
+// so half the transforms and 4 bytes per pixel of spectrum instead of 8. The
+// TPF threads of a packed row hold both rows; packed rows past the last one
+// (a CTA may hold more than are left) repeat it and store nothing.
+template <int N, int OP>
+__global__ void __launch_bounds__(row_threads(N), row_min_blocks(N, ROW_FFT)) row_pk_kernel(const PassArgs a, int nrows) {
+  pdl_wait();
+  constexpr int EPT = ept_for(N), TPF = tpf_for(N), ROWS = rows_for(N);
+  constexpr int RS = first_radix<N, FWD>();
+  constexpr int RK = last_radix<N, FWD>();
+  extern __shared__ float2 smem[];
+  const int rr = threadIdx.x / TPF, t = threadIdx.x - rr * TPF;
+  int row = blockIdx.x * ROWS + rr;
+  const bool valid = row < nrows;
+  row = (valid ? row : nrows - 1) + a.proj0 * (a.ny / 2);
+  const int proj = row / (a.ny / 2);
+  if (skip_proj(a, proj)) return;
+  const size_t rb = 2 * (size_t)row * N;  // the even row
+  const RowLayout<N, ROWS * TPF> sm{smem + rr * row_smem_len(N), 1 + rr};
+  float2 v[EPT];
+  if constexpr (OP == PKROW_FFT) {
+#pragma unroll
+    for (int j = 0; j < EPT; j++) {
+      const size_t o = rb + slot_index<N, RS>(t, j);
+      v[j] = make_float2(a.y[o], a.y[o + N]);
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < EPT; j++) v[j] = a.in[rb + pk_pos<N>(slot_index<N, RK>(t, j))];
+    fft_run<N, INV>(v, sm, t, a.tw_inv);
+  }
+  if constexpr (OP == PKROW_OUT) {
+    if (valid) {
+#pragma unroll
+      for (int j = 0; j < EPT; j++) {
+        const size_t o = rb + slot_index<N, RS>(t, j);
+        a.f_out[o] = v[j].x;
+        a.f_out[o + N] = v[j].y;
+      }
+    }
+    return;
+  }
+  if constexpr (OP == PKROW_RESID) {
+    float part = 0.f;
+#pragma unroll
+    for (int j = 0; j < EPT; j++) {
+      const size_t o = rb + slot_index<N, RS>(t, j);
+      const float e0 = a.y[o] - v[j].x, e1 = a.y[o + N] - v[j].y;
+      part = fmaf(e0, e0, fmaf(e1, e1, part));
+      v[j] = make_float2(-e0, -e1);
+    }
+    // a CTA may hold rows of two projections: each row adds its own sum
+    constexpr int W = TPF < 32 ? TPF : 32;
+    double d = valid ? (double)part : 0.0;
+    const unsigned mask = ROWS * TPF >= 32 ? 0xffffffffu : ((1u << (ROWS * TPF & 31)) - 1u);
+#pragma unroll
+    for (int o = W / 2; o > 0; o >>= 1) d += __shfl_xor_sync(mask, d, o);
+    if (valid && t % W == 0) atomicAdd(&a.acc[(size_t)proj * NACC + ACC_LOSS], d);
+  }
+  fft_run<N, FWD>(v, sm, t, a.tw_fwd);
+  if (valid) {
+#pragma unroll
+    for (int j = 0; j < EPT; j++) a.out[rb + pk_pos<N>(slot_index<N, RK>(t, j))] = v[j];
+  }
+}
+
+// ---------------------------------------------------------------------------
 // column pass
 // ---------------------------------------------------------------------------
 // C columns of one projection per tile; thread (t, c) = (tid / C, tid % C)
@@ -1041,7 +1111,7 @@ __global__ void __launch_bounds__(col2_threads(N, C), col2_min_blocks(N, C))
 // the one holding 2y' + 1 the mirror pair conj G(2y') + i conj G(2y' + 1)
 // (the partner's value comes by shuffle). Bins 0 and nx/2 are their own
 // mirrors; the first lane of the first tile leaves them (its first column is
-// computed and dropped) to col_kernel_pk_edge, which runs after this kernel.
+// computed and dropped) to pk_edge.
 // Needs the thread holding row y to hold the same slots as the one holding
 // y ^ 1, C/2 lanes apart (pk_col_ok).
 template <int N>
@@ -1049,8 +1119,86 @@ __host__ __device__ constexpr bool pk_col_ok() {
   return tpf_for(N) % 2 == 0 && (N / first_radix<N, FWD>()) % 2 == 0 && ept_for(N) % 2 == 0;
 }
 
-template <int N, int C>
-__global__ void __launch_bounds__(col2_threads(N, C), col2_min_blocks(N, C)) col_kernel_pk(const PassArgs a, int nproj) {
+// Bins 0 and nx/2 of the packed residual pass, by the first TPF threads of a CTA
+// of their own (one per projection, the last ones of col_kernel_pk's grid; as a
+// kernel after it they cost a launch more, 4 us of a small iteration): both
+// columns of the row spectrum are real (a real row's DC and
+// Nyquist bins), so they ride as one complex column W = X0 + i Xh, rebuilt from
+// packed positions 0 and nx/2 (X(2y') = Re Z(y'), X(2y' + 1) = Im Z(y')). After
+// the forward transform X0^(ky) = (W^(ky) + conj W^(-ky)) / 2 and
+// Xh^(ky) = (W^(ky) - conj W^(-ky)) / (2i) (through shared memory); each gets
+// its own bin's IOTF and F{y}, the loss (weight 1), and the two residuals go
+// back as one column g0 + i gh, whose inverse transform is G0 + i Gh (both
+// real), packed again into positions 0 and nx/2.
+template <int N, bool RES>
+__device__ __forceinline__ void pk_edge(const PassArgs& a, int proj, int t, float2* smem) {
+  constexpr int EPT = ept_for(N), TPF = tpf_for(N);
+  constexpr int RS = first_radix<N, FWD>(), RK = last_radix<N, FWD>();
+  const int hx = a.nx / 2;
+  const size_t pbase = (size_t)proj * a.ny * a.nx;
+  const size_t ldp = 2 * (size_t)a.nx;
+  const RowLayout<N, TPF> sm{smem, 1};
+  float2 v[EPT];
+#pragma unroll
+  for (int j = 0; j < EPT; j++) {
+    const int y = slot_index<N, RS>(t, j);
+    const float2 z0 = a.in[pbase + (size_t)(y >> 1) * ldp], zh = a.in[pbase + (size_t)(y >> 1) * ldp + hx];
+    v[j] = (y & 1) ? make_float2(z0.y, zh.y) : make_float2(z0.x, zh.x);
+  }
+  fft_run<N, FWD>(v, sm, t, a.tw_fwd);
+  sm.sync();  // the transform's last reads are done
+#pragma unroll
+  for (int j = 0; j < EPT; j++) sm[slot_index<N, RK>(t, j)] = v[j];
+  sm.sync();
+  float part = 0.f;
+  const float i0 = __ldg(&a.ix[0]), ih = __ldg(&a.ix[hx]);
+#pragma unroll
+  for (int j = 0; j < EPT; j++) {
+    const int ky = slot_index<N, RK>(t, j);
+    const float2 p = v[j], q = sm[ky == 0 ? 0 : N - ky];
+    const float2 x0 = make_float2(0.5f * (p.x + q.x), 0.5f * (p.y - q.y));
+    const float2 xh = make_float2(0.5f * (p.y + q.y), 0.5f * (q.x - p.x));
+    const float iy = __ldg(&a.iy[ky]);
+    const float w0 = i0 * iy, wh = ih * iy;
+    if constexpr (!RES) {
+      const float2 g0 = cscale(x0, w0 * a.scale), gh = cscale(xh, wh * a.scale);
+      v[j] = make_float2(g0.x - gh.y, g0.y + gh.x);  // g0 + i gh
+      continue;
+    }
+    const float2 y0 = a.yhat[pbase + (size_t)ky * a.nx], yh = a.yhat[pbase + (size_t)ky * a.nx + hx];
+    const float2 r0 = make_float2(fmaf(w0, x0.x, -y0.x), fmaf(w0, x0.y, -y0.y));
+    const float2 rh = make_float2(fmaf(wh, xh.x, -yh.x), fmaf(wh, xh.y, -yh.y));
+    part = fmaf(r0.x, r0.x, fmaf(r0.y, r0.y, part));
+    part = fmaf(rh.x, rh.x, fmaf(rh.y, rh.y, part));
+    const float2 g0 = cscale(r0, w0 * a.scale), gh = cscale(rh, wh * a.scale);
+    v[j] = make_float2(g0.x - gh.y, g0.y + gh.x);  // g0 + i gh
+  }
+  part *= a.scale;
+  fft_run<N, INV>(v, sm, t, a.tw_inv);  // its first write waits for the reads above
+  sm.sync();
+#pragma unroll
+  for (int j = 0; j < EPT; j++) sm[slot_index<N, RS>(t, j)] = v[j];
+  sm.sync();
+#pragma unroll
+  for (int k = 0; k < EPT / 2; k++) {
+    const int yp = t + k * TPF;
+    const float2 e = sm[2 * yp], o = sm[2 * yp + 1];
+    a.out[pbase + (size_t)yp * ldp] = make_float2(e.x, o.x);
+    a.out[pbase + (size_t)yp * ldp + hx] = make_float2(e.y, o.y);
+  }
+  if constexpr (RES) {
+    constexpr int W = TPF < 32 ? TPF : 32;
+    constexpr unsigned mask = W == 32 ? 0xffffffffu : (1u << (W & 31)) - 1u;
+    double d = (double)part;
+#pragma unroll
+    for (int o = W / 2; o > 0; o >>= 1) d += __shfl_xor_sync(mask, d, o);
+    if (t % W == 0) atomicAdd(&a.acc[proj * NACC + ACC_LOSS], d);
+  }
+}
+
+// RES = false: the IOTF filter alone, on packed rows (no F{y}, no loss).
+template <int N, int C, bool RES>
+__global__ void __launch_bounds__(col2_threads(N, C), col2_min_blocks(N, C)) col_kernel_pk(const PassArgs a, int nproj, int tile_ctas) {
   pdl_wait();
   constexpr int EPT = ept_for(N);
   constexpr int TPFC = tpf_for(N);      // threads per column pair
@@ -1072,7 +1220,12 @@ __global__ void __launch_bounds__(col2_threads(N, C), col2_min_blocks(N, C)) col
   const bool odd = (t & 1) != 0;        // this thread holds the odd rows 2y' + 1
   const ColPairLayout<N, C> sm{smem + 2 * c2};
 
-  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+  if ((int)blockIdx.x >= tile_ctas) {
+    const int proj = a.proj0 + (int)blockIdx.x - tile_ctas;
+    if (tid < TPFC && !skip_proj(a, proj)) pk_edge<N, RES>(a, proj, tid, smem);
+    return;
+  }
+  for (int tile = blockIdx.x; tile < ntiles; tile += tile_ctas) {
     const int proj = a.proj0 + tile / tiles_per_proj;
     const int c0 = (tile % tiles_per_proj) * C;
     if (skip_proj(a, proj)) continue;  // uniform over the CTA
@@ -1090,7 +1243,7 @@ __global__ void __launch_bounds__(col2_threads(N, C), col2_min_blocks(N, C)) col
     __syncthreads();
 
     const int kx = c0 + 2 * c2;      // bins kx, kx + 1 (mirrors nx - kx, nx - kx - 1)
-    const bool edge = kx == 0;       // bin 0 (and nx/2): col_kernel_pk_edge's
+    const bool edge = kx == 0;       // bin 0 (and nx/2): pk_edge's
     {
       // X(2y') = (Z + conj Zm) / 2 and X(2y' + 1) = (Z - conj Zm) / (2i) of
       // both columns, from the front (Z) and mirror (Zm) rows y'
@@ -1126,6 +1279,11 @@ __global__ void __launch_bounds__(col2_threads(N, C), col2_min_blocks(N, C)) col
     for (int j = 0; j < EPT; j++) {
       const int ky = slot_index<N, RK>(t, j);
       const float iy = __ldg(&a.iy[ky]);
+      if constexpr (!RES) {
+        v[j] = cscale(v[j], ia * iy * a.scale);
+        u[j] = cscale(u[j], ib * iy * a.scale);
+        continue;
+      }
       const float4 yh = *reinterpret_cast<const float4*>(a.yhat + pbase + (size_t)ky * a.nx + kx);
       const float wa = ia * iy, wb = ib * iy;
       const float2 ra = make_float2(fmaf(wa, v[j].x, -yh.x), fmaf(wa, v[j].y, -yh.y));
@@ -1154,78 +1312,10 @@ __global__ void __launch_bounds__(col2_threads(N, C), col2_min_blocks(N, C)) col
       else
         *reinterpret_cast<float4*>(dst) = o;
     }
-    block_reduce_add<1>(part, a.acc, proj * NACC + ACC_LOSS, smem);
+    if constexpr (RES) block_reduce_add<1>(part, a.acc, proj * NACC + ACC_LOSS, smem);
     __syncthreads();  // the buffer is refilled by the next tile's copy
   }
   cp_async_wait<0>();
-}
-
-// Bins 0 and nx/2 of the packed residual pass, one CTA per projection, after
-// col_kernel_pk: both columns of the row spectrum are real (a real row's DC and
-// Nyquist bins), so they ride as one complex column W = X0 + i Xh, rebuilt from
-// packed positions 0 and nx/2 (X(2y') = Re Z(y'), X(2y' + 1) = Im Z(y')). After
-// the forward transform X0^(ky) = (W^(ky) + conj W^(-ky)) / 2 and
-// Xh^(ky) = (W^(ky) - conj W^(-ky)) / (2i) (through shared memory); each gets
-// its own bin's IOTF and F{y}, the loss (weight 1), and the two residuals go
-// back as one column g0 + i gh, whose inverse transform is G0 + i Gh (both
-// real), packed again into positions 0 and nx/2.
-template <int N>
-__global__ void __launch_bounds__(tpf_for(N)) col_kernel_pk_edge(const PassArgs a) {
-  pdl_wait();
-  constexpr int EPT = ept_for(N), TPF = tpf_for(N);
-  constexpr int RS = first_radix<N, FWD>(), RK = last_radix<N, FWD>();
-  extern __shared__ float2 smem[];
-  const int proj = a.proj0 + blockIdx.x;
-  if (skip_proj(a, proj)) return;
-  const int t = threadIdx.x;
-  const int hx = a.nx / 2;
-  const size_t pbase = (size_t)proj * a.ny * a.nx;
-  const size_t ldp = 2 * (size_t)a.nx;
-  const RowLayout<N, TPF> sm{smem, 1};
-  float2 v[EPT];
-#pragma unroll
-  for (int j = 0; j < EPT; j++) {
-    const int y = slot_index<N, RS>(t, j);
-    const float2 z0 = a.in[pbase + (size_t)(y >> 1) * ldp], zh = a.in[pbase + (size_t)(y >> 1) * ldp + hx];
-    v[j] = (y & 1) ? make_float2(z0.y, zh.y) : make_float2(z0.x, zh.x);
-  }
-  fft_run<N, FWD>(v, sm, t, a.tw_fwd);
-  sm.sync();  // the transform's last reads are done
-#pragma unroll
-  for (int j = 0; j < EPT; j++) sm[slot_index<N, RK>(t, j)] = v[j];
-  sm.sync();
-  float part[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-  const float i0 = __ldg(&a.ix[0]), ih = __ldg(&a.ix[hx]);
-#pragma unroll
-  for (int j = 0; j < EPT; j++) {
-    const int ky = slot_index<N, RK>(t, j);
-    const float2 p = v[j], q = sm[ky == 0 ? 0 : N - ky];
-    const float2 x0 = make_float2(0.5f * (p.x + q.x), 0.5f * (p.y - q.y));
-    const float2 xh = make_float2(0.5f * (p.y + q.y), 0.5f * (q.x - p.x));
-    const float iy = __ldg(&a.iy[ky]);
-    const float w0 = i0 * iy, wh = ih * iy;
-    const float2 y0 = a.yhat[pbase + (size_t)ky * a.nx], yh = a.yhat[pbase + (size_t)ky * a.nx + hx];
-    const float2 r0 = make_float2(fmaf(w0, x0.x, -y0.x), fmaf(w0, x0.y, -y0.y));
-    const float2 rh = make_float2(fmaf(wh, xh.x, -yh.x), fmaf(wh, xh.y, -yh.y));
-    part[0] = fmaf(r0.x, r0.x, fmaf(r0.y, r0.y, part[0]));
-    part[0] = fmaf(rh.x, rh.x, fmaf(rh.y, rh.y, part[0]));
-    const float2 g0 = cscale(r0, w0 * a.scale), gh = cscale(rh, wh * a.scale);
-    v[j] = make_float2(g0.x - gh.y, g0.y + gh.x);  // g0 + i gh
-  }
-  part[0] *= a.scale;
-  fft_run<N, INV>(v, sm, t, a.tw_inv);  // its first write waits for the reads above
-  sm.sync();
-#pragma unroll
-  for (int j = 0; j < EPT; j++) sm[slot_index<N, RS>(t, j)] = v[j];
-  sm.sync();
-#pragma unroll
-  for (int k = 0; k < EPT / 2; k++) {
-    const int yp = t + k * TPF;
-    const float2 e = sm[2 * yp], o = sm[2 * yp + 1];
-    a.out[pbase + (size_t)yp * ldp] = make_float2(e.x, o.x);
-    a.out[pbase + (size_t)yp * ldp + hx] = make_float2(e.y, o.y);
-  }
-  block_reduce_add<1>(part, a.acc, proj * NACC + ACC_LOSS, smem);
 }
 
 // ---------------------------------------------------------------------------
@@ -1655,6 +1745,19 @@ cudaError_t launch_row(const PassArgs& a, int nproj, cudaStream_t s) {
   return launch_pass(row_kernel<N, OP>, dim3((unsigned)(nrows / ROWS)), dim3(row_threads(N)), row_smem_bytes(N), s, a.pdl, a);
 }
 
+template <int N, int OP>
+cudaError_t prep_row_pk() {
+  return cudaFuncSetAttribute(row_pk_kernel<N, OP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)row_smem_bytes(N));
+}
+// packed row pass over the ny/2 packed rows of nproj projections starting at a.proj0
+template <int N, int OP>
+cudaError_t launch_row_pk(const PassArgs& a, int nproj, cudaStream_t s) {
+  constexpr int ROWS = rows_for(N);
+  const int nrows = nproj * (a.ny / 2);
+  return launch_pass(row_pk_kernel<N, OP>, dim3((unsigned)((nrows + ROWS - 1) / ROWS)), dim3(row_threads(N)),
+                     row_smem_bytes(N), s, a.pdl, a, nrows);
+}
+
 // column-pass shape variants: tile width C, pipelined or not
 template <int N, int OP, int C, int PIPE>
 struct ColShape {
@@ -1744,17 +1847,18 @@ template <int N, int OP, int C, int PIPE>
 int ColShape<N, OP, C, PIPE>::resident = 1;
 
 
-// Packed residual shapes (COL_RESID_PK): persistent, one staged buffer, column
-// pairs (described like the single-buffered pair shapes, pipe code 4).
-template <int N, int C>
+// Packed residual shapes (COL_RESID_PK), and the packed IOTF filter (RES =
+// false) in the same shapes: persistent, one staged buffer, column pairs
+// (described like the single-buffered pair shapes, pipe code 4).
+template <int N, int C, bool RES>
 struct PkShape {
   static int resident;
   static cudaError_t prep() {
     constexpr size_t SM = col_smem_bytes(N, C);
-    cudaError_t e = cudaFuncSetAttribute(col_kernel_pk<N, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM);
+    cudaError_t e = cudaFuncSetAttribute(col_kernel_pk<N, C, RES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM);
     if (e != cudaSuccess) return e;
     int r = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, col_kernel_pk<N, C>, col2_threads(N, C), SM);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, col_kernel_pk<N, C, RES>, col2_threads(N, C), SM);
     resident = r > 0 ? r : 1;
     return e;
   }
@@ -1762,16 +1866,13 @@ struct PkShape {
     const long long ntiles = (long long)nproj * (a.nx / 2 / C);
     const long long slots = (long long)device_sms() * resident;
     const int grid = (int)(ntiles < slots ? ntiles : slots);
-    cudaError_t e = launch_pass(col_kernel_pk<N, C>, dim3(grid), dim3(col2_threads(N, C)), col_smem_bytes(N, C), s,
-                                a.pdl, a, nproj);
-    if (e != cudaSuccess) return e;
-    // then bins 0 and nx/2 of every projection
-    return launch_pass(col_kernel_pk_edge<N>, dim3(nproj), dim3(tpf_for(N)), row_smem_len(N) * sizeof(float2), s, a.pdl,
-                       a);
+    // the tiles, then a CTA for bins 0 and nx/2 of every projection
+    return launch_pass(col_kernel_pk<N, C, RES>, dim3(grid + nproj), dim3(col2_threads(N, C)), col_smem_bytes(N, C), s,
+                       a.pdl, a, nproj, grid);
   }
 };
-template <int N, int C>
-int PkShape<N, C>::resident = 1;
+template <int N, int C, bool RES>
+int PkShape<N, C, RES>::resident = 1;
 
 // whole warps (the output pairs rows by shuffle), even chunk split; a plan
 // takes a shape only where C divides nx/2 (pk_fits)
@@ -1786,8 +1887,10 @@ template <int N, int C>
 void add_pk_variant(LengthKernels& k) {
   if constexpr (pk_shape_ok<N, C>()) {
     int& n = k.ncolv[COL_RESID_PK];
-    if (n < MAX_COL_VARIANTS)
-      k.colv[COL_RESID_PK][n++] = {PkShape<N, C>::launch, PkShape<N, C>::prep, C, 4, PWF_SCHED_VARIANT};
+    if (n < MAX_COL_VARIANTS) {
+      k.iotf_pk[n] = {PkShape<N, C, false>::launch, PkShape<N, C, false>::prep, C, 4, PWF_SCHED_VARIANT};
+      k.colv[COL_RESID_PK][n++] = {PkShape<N, C, true>::launch, PkShape<N, C, true>::prep, C, 4, PWF_SCHED_VARIANT};
+    }
   }
 }
 
@@ -1952,6 +2055,11 @@ LengthKernels make_length_kernels() {
   PWF_ROW(ROW_NESTEROV_FFT) PWF_ROW(ROW_NESTEROV) PWF_ROW(ROW_GRADT) PWF_ROW(ROW_MODE_INT) PWF_ROW(ROW_MODE_VG)
   PWF_ROW(ROW_INTENSITY_PK) PWF_ROW(ROW_MUL_V_PK)
 #undef PWF_ROW
+#define PWF_ROW_PK(OP)                  \
+  k.row_pk[OP] = launch_row_pk<N, OP>;  \
+  k.row_pk_prep[OP] = prep_row_pk<N, OP>;
+  PWF_ROW_PK(PKROW_FFT) PWF_ROW_PK(PKROW_OUT) PWF_ROW_PK(PKROW_RESID)
+#undef PWF_ROW_PK
   add_col_op<N, COL_Q>(k);
   add_col_op<N, COL_IOTF>(k);
   add_col_op<N, COL_RESID_IOTF2>(k);
