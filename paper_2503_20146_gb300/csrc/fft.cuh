@@ -3,7 +3,7 @@
 // Every Filter of Algorithm S2 (F^-1{F{x} W}) is evaluated as a row transform
 // and a column transform of a complex64 field. This header holds the pieces
 // shared by the row and column kernels:
-//   * complex helpers and radix-2/3/4/8/16 DFT butterflies (written from the
+//   * complex helpers and radix-2/3/4/8/12/16/24/32 DFT butterflies (written from the
 //     DFT definition X_k = sum_j x_j exp(s 2 pi i j k / R), s = -1 forward);
 //   * a compile-time radix schedule per transform length N (N = 2^a 3^b);
 //   * a self-sorting (Stockham) stage runner: stage 0 takes its inputs from
@@ -376,7 +376,8 @@ struct Sched {
 };
 
 // The alternative schedules (set 1): the same stages in another order where
-// that keeps the values per thread, or smaller radices where it cuts them
+// that keeps the values per thread, or smaller radices where it cuts them (1024
+// with 16 instead of 32 values)
 // (fewer registers per transform, more warps per SM, shorter dependent chains
 // per thread, at the price of more exchanges: 128 = 4.4.4.2 runs one
 // transform per warp with four values per thread; 768 and 1536 keep 12 values

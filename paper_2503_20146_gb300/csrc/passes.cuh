@@ -248,7 +248,7 @@ __device__ __forceinline__ void row_body(const PassArgs& a, long long row, int t
   // side input before they store: a store may alias the next load as far as
   // the compiler knows, which would leave one load in flight at a time. On 180
   // x 1024^2 (ms per launch): row_grad_pack 1.78 -> 1.18, row_nesterov_fft 2.04
-  // -> 1.74; on 24 x 1024^2 row_mode_int 0.162 -> 0.094, col_mode_back 0.187 ->
+  // -> 1.72; on 24 x 1024^2 row_mode_int 0.162 -> 0.094, col_mode_back 0.187 ->
   // 0.139, row_exp_fft 0.211 -> 0.072 (with sincos_acc).
   constexpr int BL = EPT % 8 == 0 ? 8 : EPT;
 
@@ -437,7 +437,7 @@ __device__ __forceinline__ void row_body(const PassArgs& a, long long row, int t
     }
   } else if constexpr (OP == ROW_NESTEROV_FFT || OP == ROW_NESTEROV) {
     const float beta = *a.beta;
-    constexpr int BN = EPT % 4 == 0 ? 4 : EPT;
+    constexpr int BN = EPT >= 32 ? 8 : EPT % 4 == 0 ? 4 : EPT;  // three side inputs: what the registers hold
 #pragma unroll
     for (int j0 = 0; j0 < EPT; j0 += BN) {
      float2 ps[BN], ph[BN];
@@ -1983,21 +1983,29 @@ void add_col_variant(LengthKernels& k) {
 
 template <int N, int OP>
 void add_col_op(LengthKernels& k) {
-  // first entry = default before tuning
-  add_col_variant<N, OP, (N >= 1024 ? 8 : 16), 1>(k);
-  add_col_variant<N, OP, 16, 0>(k);
+  // first entry = default before tuning. Left out where they never came near the
+  // fastest: transposed tiles and 4-column TMA tiles from length 1024 on, wide
+  // tiles with 32 values per thread (they spill).
+  constexpr bool LONG = N >= 1024, WIDE = ept_for(N) >= 32;
+  constexpr int FIRST = !WIDE ? 0 : OP == COL_PRECOND_REG ? 1 : OP == COL_RESID_IOTF2 ? 2 : 0;
+  if constexpr (FIRST == 1) add_col_variant<N, OP, 4, 0>(k);
+  if constexpr (FIRST == 2) add_col_variant<N, OP, 4, 1>(k);
+  add_col_variant<N, OP, (LONG ? 8 : 16), 1>(k);
+  if constexpr (!WIDE) add_col_variant<N, OP, 16, 0>(k);
   add_col_variant<N, OP, 8, 0>(k);
-  add_col_variant<N, OP, 4, 0>(k);
-  add_col_variant<N, OP, 4, 1>(k);
-  if constexpr (N < 1024) add_col_variant<N, OP, 8, 1>(k);
-  add_col_variant<N, OP, 8, 2>(k);
-  add_col_variant<N, OP, 4, 2>(k);
-  add_col_variant<N, OP, 8, 3>(k);
+  if constexpr (FIRST != 1) add_col_variant<N, OP, 4, 0>(k);
+  if constexpr (FIRST != 2) add_col_variant<N, OP, 4, 1>(k);
+  if constexpr (!LONG) add_col_variant<N, OP, 8, 1>(k);
+  if constexpr (!LONG) {
+    add_col_variant<N, OP, 8, 2>(k);
+    add_col_variant<N, OP, 4, 2>(k);
+  }
+  if constexpr (!WIDE) add_col_variant<N, OP, 8, 3>(k);
   add_col_variant<N, OP, 8, 4>(k);
-  add_col_variant<N, OP, 16, 4>(k);
+  if constexpr (!WIDE) add_col_variant<N, OP, 16, 4>(k);
   add_col_variant<N, OP, 4, 4>(k);
   add_col_variant<N, OP, 8, 5>(k);
-  add_col_variant<N, OP, 4, 5>(k);
+  if constexpr (!LONG) add_col_variant<N, OP, 4, 5>(k);
   add_col_variant<N, OP, 8, 7>(k);
   add_col_variant<N, OP, 4, 7>(k);
 }
@@ -2068,7 +2076,7 @@ LengthKernels make_length_kernels() {
   add_col_op<N, COL_IFFT>(k);
   add_pk_variant<N, 8>(k);  // first entry = default before tuning (fits every nx >= 16)
   add_pk_variant<N, 4>(k);
-  add_pk_variant<N, 16>(k);
+  if constexpr (ept_for(N) < 32) add_pk_variant<N, 16>(k);
   add_mode_op<N, CM_FWD>(k);
   add_mode_op<N, CM_BACK>(k);
   return k;
