@@ -608,7 +608,7 @@ def run_fbp(P, S, torch, dev, stream, psi, w, reps=3):
     ms = e0.elapsed_time(e1) / reps
     updates = float(n_ang) * ny * nx * nx
     out = {"ms": ms, "voxel_angle_updates_per_s": updates / (ms / 1e3), "volume": [ny, nx, nx],
-           "angles": n_ang, "note": "includes the host-side ramp and angle tables (synchronous copies)"}
+           "angles": n_ang, "note": "includes the ramp, twiddle and angle tables, made on the device per call"}
     del vol, ws
     return out
 

@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(BP_TX * BP_TY)
 // order of visits nearer to the detector position (0.39 taps) measured the
 // same 9.0. Four slices per lane (8 warps, 190 registers) measured 8.9, two
 // (16 warps) 9.8; twelve warps of 4 x 4 patches 8.7, with overhanging tiles.
-// Whole call, 180 x 1024 x 1024: 162.7 -> 71.9 ms (one thread per voxel reading
+// Whole call, 180 x 1024 x 1024: 162.7 -> 71.6 ms (one thread per voxel reading
 // records through the L1, and 13 ms of host cosines).
 // Each stage of two angles is copied by cp.async while the ones before it are
 // used; a stage holds at most ROWS rows, the columns under the tile's diagonal.
