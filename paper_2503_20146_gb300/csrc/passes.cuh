@@ -1819,14 +1819,17 @@ struct ColShape {
         return launch_pass(col_kernel_pipe2<N, OP, C, 2>, dim3(grid), dim3(col2_threads(N, C)), colp_smem_bytes(N, C), s,
                            a.pdl, a, nproj);
       else if constexpr (PIPE == 4) {
-        PassArgs b = a;  // with a tensor map of the field, the kernel prefetches each next tile into L2
-        b.l2pf = encode_field_tmap(&b.tmap, a.in, a.proj0 + nproj, a.ny, a.nx, C) ? 1 : 0;
+        // with a tensor map of the field, the kernel prefetches each next tile into
+        // L2 (a launch of one wave has no next tile: encoding the map, 1 us on the
+        // host, is left out)
+        PassArgs b = a;
+        b.l2pf = ntiles > slots && encode_field_tmap(&b.tmap, a.in, a.proj0 + nproj, a.ny, a.nx, C) ? 1 : 0;
         return launch_pass(col_kernel_pipe2<N, OP, C, 1>, dim3(grid), dim3(col2_threads(N, C)), col_smem_bytes(N, C), s,
                            a.pdl, b, nproj);
       } else if constexpr (PIPE == 7) {
         PassArgs b = a;
         CUtensorMap m2{};
-        b.l2pf = encode_field_tmap(&b.tmap, a.in, a.proj0 + nproj, a.ny, a.nx, C) ? 1 : 0;
+        b.l2pf = ntiles > slots && encode_field_tmap(&b.tmap, a.in, a.proj0 + nproj, a.ny, a.nx, C) ? 1 : 0;
         if (OP == COL_PRECOND_REG && b.l2pf) b.l2pf = encode_field_tmap(&m2, a.aux_in, a.proj0 + nproj, a.ny, a.nx, C) ? 1 : 0;
         return launch_pass(col_kernel_pipe<N, OP, C, 1>, dim3(grid), dim3(col_threads(N, C)), col_smem_bytes(N, C), s,
                            a.pdl, b, nproj, m2);
