@@ -1901,14 +1901,17 @@ void add_pk_variant(LengthKernels& k) {
 // adjacent columns. The first one registered is the default before tuning:
 // 8 columns per tile from length 1024 on (4 where 8 would exceed 512
 // threads), else 16; the pair kernel where a transform has 16 values per
-// thread and at most 64 threads.
+// thread and at most 64 threads. A CTA has at least a warp, but for length 16:
+// one thread per transform, so that its widest tile (16 columns, the narrowest
+// field) has 16 threads.
 __host__ __device__ constexpr int colmode_c(int n) { return n >= 1024 ? (tpf_for(n) * 8 <= 512 ? 8 : 4) : 16; }
 __host__ __device__ constexpr bool colmode_pair(int n) { return ept_for(n) == 16 && tpf_for(n) <= 64 && n >= 128; }
 
 template <int N, int MOP, int C, bool PAIR>
 constexpr bool mode_shape_ok() {
   constexpr int th = PAIR ? col2_threads(N, C) : col_threads(N, C);
-  return th >= 32 && th <= 512 && col_smem_bytes(N, C) <= 200 * 1024 && N % C == 0 &&
+  constexpr int least = !PAIR && C == 16 ? 16 : 32;
+  return th >= least && th <= 512 && col_smem_bytes(N, C) <= 200 * 1024 && N % C == 0 &&
          (!PAIR || (C >= 4 && ept_for(N) <= 16));
 }
 
@@ -2080,6 +2083,9 @@ LengthKernels make_length_kernels() {
   add_pk_variant<N, 8>(k);  // first entry = default before tuning (fits every nx >= 16)
   add_pk_variant<N, 4>(k);
   if constexpr (ept_for(N) < 32) add_pk_variant<N, 16>(k);
+  static_assert(mode_shape_ok<N, CM_FWD, 16, false>() || mode_shape_ok<N, CM_FWD, 8, false>() ||
+                    mode_shape_ok<N, CM_FWD, 4, false>(),
+                "every length needs a shape of the mode column passes");
   add_mode_op<N, CM_FWD>(k);
   add_mode_op<N, CM_BACK>(k);
   return k;
