@@ -1110,8 +1110,9 @@ __global__ void __launch_bounds__(col2_threads(N, C), col2_min_blocks(N, C))
 // residual: the thread holding row 2y' the front pair G(2y') + i G(2y' + 1),
 // the one holding 2y' + 1 the mirror pair conj G(2y') + i conj G(2y' + 1)
 // (the partner's value comes by shuffle). Bins 0 and nx/2 are their own
-// mirrors; the first lane of the first tile leaves them (its first column is
-// computed and dropped) to pk_edge.
+// mirrors: no tile reads or writes their positions 0 and nx/2, which pk_edge
+// transforms in a CTA of the same launch. The first lane of the first tile holds
+// a column of zeros in their place and drops it.
 // Needs the thread holding row y to hold the same slots as the one holding
 // y ^ 1, C/2 lanes apart (pk_col_ok).
 template <int N>
@@ -1235,8 +1236,16 @@ __global__ void __launch_bounds__(col2_threads(N, C), col2_min_blocks(N, C)) col
       const int q = tid + k * NT;
       const int half = q / CHUNKS, qq = q - half * CHUNKS;
       const int row = qq / (C / 2), pr = qq % (C / 2);
-      cp_async16(smem + col_row<N>(half * H + row, C) * C + 2 * pr,
-                 a.in + pbase + (size_t)row * ldp + (half ? hx : 0) + c0 + 2 * pr);
+      float2* dst = smem + col_row<N>(half * H + row, C) * C + 2 * pr;
+      const float2* src = a.in + pbase + (size_t)row * ldp + (half ? hx : 0) + c0 + 2 * pr;
+      if (c0 == 0 && pr == 0) {
+        // positions 0 and nx/2 are pk_edge's: its CTA writes them while this one
+        // runs, so they are not read, and the column they would make is zero
+        dst[0] = make_float2(0.f, 0.f);
+        cp_async8(dst + 1, src + 1);
+      } else {
+        cp_async16(dst, src);
+      }
     }
     cp_async_commit();
     cp_async_wait<0>();
