@@ -125,19 +125,36 @@ __device__ __forceinline__ float2 cadd_i(float2 a, float2 b) {
   else return cadd<false>(a, mul_si<DIR>(b));
 }
 
+// The butterflies' constants. The FP32 pairs nearest to exp(i pi/8) and
+// exp(i pi/16) are both 3e-8 short of modulus 1, sqrt(3)/2 is 2e-8 short of its
+// value, and a constant takes part in every row and column alike: the losses of a
+// transform and its inverse add up over the filters of a pass chain to a
+// common factor of the modelled intensity. The inverse therefore takes the next
+// FP32 numbers above, as much too long, so that a constant and its counterpart
+// cancel (gain of transform and inverse, nearest numbers -> these: 1024 -8.3e-8 ->
+// -1.9e-8, 2048 -6.6e-8 -> -3.2e-8, 1536 -7.1e-8 -> -4.8e-8, 256 -5.1e-8 -> -1.9e-8; rms
+// error at 1024 1.72e-7 -> 1.48e-7, with 16.8.8 and the nearest numbers 1.56e-7).
+// sqrt(1/2), 1.7e-8 short, has no such counterpart (the next number is 6.7e-8
+// too long), nor exp(3 i pi/16), 0.7e-8 short.
+template <int DIR>
+struct Trig {
+  static constexpr float cos_8 = DIR == FWD ? 0.923879504f : 0.923879564f;   // pi/8
+  static constexpr float sin_8 = DIR == FWD ? 0.382683426f : 0.382683456f;
+  static constexpr float cos_16 = DIR == FWD ? 0.980785251f : 0.98078531f;   // pi/16
+  static constexpr float sin_16 = DIR == FWD ? 0.195090324f : 0.195090339f;
+  static constexpr float cos_316 = 0.83146961230254524f;                     // 3 pi/16
+  static constexpr float sin_316 = 0.55557023301960218f;
+  static constexpr float half_sqrt3 = DIR == FWD ? 0.866025388f : 0.866025448f;
+};
+
 // exp(s 2 pi i m / 16) for the compile-time exponent m
 template <int DIR, int M>
 __device__ __forceinline__ float2 w16() {
   constexpr int m = M & 15;
+  constexpr float c1 = Trig<DIR>::cos_8, s1 = Trig<DIR>::sin_8, h = 0.70710678118654752f;
   // cos and sin of m*pi/8 for m = 0..15
-  constexpr float C[16] = {1.0f, 0.92387953251128674f, 0.70710678118654752f, 0.38268343236508977f,
-                           0.0f, -0.38268343236508977f, -0.70710678118654752f, -0.92387953251128674f,
-                           -1.0f, -0.92387953251128674f, -0.70710678118654752f, -0.38268343236508977f,
-                           0.0f, 0.38268343236508977f, 0.70710678118654752f, 0.92387953251128674f};
-  constexpr float S[16] = {0.0f, 0.38268343236508977f, 0.70710678118654752f, 0.92387953251128674f,
-                           1.0f, 0.92387953251128674f, 0.70710678118654752f, 0.38268343236508977f,
-                           0.0f, -0.38268343236508977f, -0.70710678118654752f, -0.92387953251128674f,
-                           -1.0f, -0.92387953251128674f, -0.70710678118654752f, -0.38268343236508977f};
+  constexpr float C[16] = {1.0f, c1, h, s1, 0.0f, -s1, -h, -c1, -1.0f, -c1, -h, -s1, 0.0f, s1, h, c1};
+  constexpr float S[16] = {0.0f, s1, h, c1, 1.0f, c1, h, s1, 0.0f, -s1, -h, -c1, -1.0f, -c1, -h, -s1};
   return make_float2(C[m], DIR == FWD ? -S[m] : S[m]);
 }
 
@@ -163,7 +180,7 @@ __device__ __forceinline__ void dft2(float2* x) {
 
 template <bool PK, int DIR>
 __device__ __forceinline__ void dft3(float2* x) {
-  constexpr float H = 0.86602540378443865f;  // sqrt(3)/2
+  constexpr float H = Trig<DIR>::half_sqrt3;
   float2 s = cadd<PK>(x[1], x[2]);
   float2 d = csub<PK>(x[1], x[2]);
   float2 m = make_float2(fmaf(-0.5f, s.x, x[0].x), fmaf(-0.5f, s.y, x[0].y));
@@ -245,12 +262,10 @@ __device__ __forceinline__ float2 twm32(float2 a) {
     return twm16<PK, DIR, m / 2>(a);
   } else {
     // cos and sin of m*pi/16 for odd m
-    constexpr double PI = 3.14159265358979323846;
-    constexpr float c1 = 0.98078528040323043f, s1 = 0.19509032201612825f;  // pi/16
-    constexpr float c3 = 0.83146961230254524f, s3 = 0.55557023301960218f;  // 3 pi/16
-    constexpr float c5 = 0.55557023301960218f, s5 = 0.83146961230254524f;  // 5 pi/16
-    constexpr float c7 = 0.19509032201612825f, s7 = 0.98078528040323043f;  // 7 pi/16
-    (void)PI;
+    constexpr float c1 = Trig<DIR>::cos_16, s1 = Trig<DIR>::sin_16;    // pi/16
+    constexpr float c3 = Trig<DIR>::cos_316, s3 = Trig<DIR>::sin_316;  // 3 pi/16
+    constexpr float c5 = s3, s5 = c3;                                  // 5 pi/16
+    constexpr float c7 = s1, s7 = c1;                                  // 7 pi/16
     // reduce m to the first quadrant: angle = m pi / 16
     constexpr int q = m / 8, r = m % 8;  // m = 8q + r, r odd
     constexpr float cr = r == 1 ? c1 : r == 3 ? c3 : r == 5 ? c5 : c7;
