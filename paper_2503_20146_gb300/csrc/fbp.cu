@@ -24,7 +24,6 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
-#include <vector>
 
 #include "../../include/pwf.h"
 #include "device_tables.cuh"
@@ -78,6 +77,16 @@ __global__ void k_fbp_tables(const __grid_constant__ AnglePart part, int first, 
   }
   for (int o = 16; o > 0; o >>= 1) h += __shfl_xor_sync(0xffffffffu, h, o);
   if (lane == 0) ramp[m] = (float)((0.25 + h) / L);
+}
+
+// Dynamic shared memory above 48 KB has to be allowed for a kernel, in each
+// context that runs it (a process may call from several devices): pwf_fbp has no
+// plan that would do it once, so every call does, with the same number each
+// time (the most the kernel can ask for), whichever thread comes first.
+template <class K>
+cudaError_t allow_shared(K* kernel, size_t bytes) {
+  return bytes <= 48 * 1024 ? cudaSuccess
+                            : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
 // One detector row per TPF threads. The nx samples are zero-padded to L = 2 nx (so that the circular convolution of
@@ -157,9 +166,7 @@ cudaError_t launch_filter_form(const float2* in, float2* out, const float* ramp,
   const long long blocks = TILES ? (long long)n_angles * ((ny + ROWS - 1) / ROWS)
                                  : ((long long)n_angles * ny + ROWS - 1) / ROWS;
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-  static const cudaError_t attr = cudaFuncSetAttribute(
-      fbp_filter_kernel<L, TILES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)row_smem_bytes(L));
-  if (attr != cudaSuccess) return attr;
+  if (const cudaError_t e = allow_shared(fbp_filter_kernel<L, TILES>, row_smem_bytes(L)); e != cudaSuccess) return e;
   fbp_filter_kernel<L, TILES>
       <<<(unsigned)blocks, row_threads(L), row_smem_bytes(L), s>>>(in, out, ramp, twf, twi, n_angles, ny, tile_slices(ny));
   return cudaGetLastError();
@@ -483,9 +490,7 @@ template <int H>
 cudaError_t launch_tiles(const float2* q, float2* vol, const double2* cs, int n_angles, int ny, int nx, float scale,
                          cudaStream_t s) {
   using S = TileShape<H>;
-  static const cudaError_t attr = cudaFuncSetAttribute(
-      fbp_backproject_tiles<H>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::bytes(PWF_FBP_MAX_ANGLES));
-  if (attr != cudaSuccess) return attr;
+  if (const cudaError_t e = allow_shared(fbp_backproject_tiles<H>, S::bytes(PWF_FBP_MAX_ANGLES)); e != cudaSuccess) return e;
   const dim3 grid(nx / BT, nx / S::TZ, (ny + S::SLICES - 1) / S::SLICES);  // nx is a multiple of 16
   fbp_backproject_tiles<H><<<grid, S::WARPS * 32, S::bytes(n_angles), s>>>(q, vol, cs, n_angles, ny, nx, scale,
                                                                            ((uintptr_t)vol & 15) == 0);
