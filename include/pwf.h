@@ -373,9 +373,9 @@ size_t pwf_plan_describe(const pwf_plan* plan, char* buf, size_t len);
  * accumulated). Each pass's shapes cover both radix schedules of the length
  * where it has two. pwf_plan_column_shapes returns how many shapes the plan's
  * column length was built with (-1 on a bad argument);
- * pwf_plan_set_column_shape forces one (0-based), replacing the tuned choice
- * (for pass 6 it also turns the packed forward model, gradient and VJP on for
- * a plan too small for them). */
+ * pwf_plan_set_column_shape forces one (0-based), replacing the tuned choice.
+ * Pass 6's shape is also that of the packed IOTF filter, which the forward
+ * model, gradient and VJP of a plan from 2^20 pixels on take. */
 int32_t pwf_plan_column_shapes(const pwf_plan* plan, int32_t pass);
 pwf_status pwf_plan_set_column_shape(pwf_plan* plan, int32_t pass, int32_t shape);
 pwf_status pwf_profile_iteration(pwf_plan* plan, const float* y, const void* t, void* psi, int32_t iters,

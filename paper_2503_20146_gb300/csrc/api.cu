@@ -403,7 +403,6 @@ struct pwf_plan {
   const LengthKernels* krow = nullptr;  // length nx
   const LengthKernels* kcol = nullptr;  // length ny
   int colsel[NUM_COL_OPS] = {};  // chosen column-pass shape per op
-  bool pk_asked = false;         // a packed-residual shape was set by the caller
   float coltime[NUM_COL_OPS][MAX_COL_VARIANTS] = {};  // tuning times (ms per launch)
   int modesel[2] = {0, 0};                              // chosen mode column-pass shape (CM_FWD, CM_BACK)
   float modetime[2][MAX_MODE_VARIANTS] = {};            // their tuning times
@@ -949,13 +948,24 @@ bool packed_resid(const pwf_plan* p) {
          shape_fits(p, COL_RESID_PK, p->kcol->colv[COL_RESID_PK][p->colsel[COL_RESID_PK]]);
 }
 // The forward model, gradient and VJP carry their real fields (|v|^2, f, the
-// residual, the cotangent) packed too, from 2^20 pixels on (or when a packed
-// shape was asked for): half the column transforms and of the bytes, but
-// longer chains per CTA, which small launches do not hide. Unpacked / packed, us
-// per forward model: 9 x 96 x 768 34 / 39, 512^2 26 / 26, 1024^2 44 / 46, 4 x 512^2 41 /
-// 38, 2048^2 141 / 129; gradient 81 / 91, 68 / 68, 114 / 116, 100 / 93, 321 / 295.
+// residual, the cotangent) packed too, from 2^20 pixels in the batch on: half the
+// column transforms and half the bytes, but longer chains per CTA, which small
+// launches do not hide. Unpacked / packed, us per forward model and gradient:
+//   below the line  512^2            26 / 26    71 / 72
+//                   9 x 96 x 768     34 / 38    83 / 89
+//   at it (2^20)    1024^2           43 / 44   112 / 111
+//                   4 x 512^2        41 / 38    99 / 93
+//                   16 x 256^2       32 / 33    79 / 81
+//                   512 x 2048       44 / 41   116 / 108
+//                   2048 x 512       46 / 48   118 / 123
+//   above           8 x 512^2        65 / 60   151 / 140
+//                   4 x 1024^2      120 / 120  270 / 261
+//                   2048^2          142 / 130  322 / 299
+//                   2 x 2048^2      264 / 238  579 / 527
+// At the line itself the two differ by up to 7 % either way, by no rule on
+// lengths, tiles or batch; from 2^22 on the packed form is never slower.
 bool packed_real(const pwf_plan* p) {
-  return packed_resid(p) && (p->pk_asked || (long long)p->d.batch * p->d.ny * p->d.nx >= 1ll << 20);
+  return packed_resid(p) && (long long)p->d.batch * p->d.ny * p->d.nx >= 1ll << 20;
 }
 
 // one fused iteration (or the body of pwf_step): X must hold F_row{exp psi}
@@ -2295,8 +2305,7 @@ pwf_status pwf_plan_set_column_shape(pwf_plan* p, int32_t pass, int32_t shape) {
     return fail(p, PWF_ERR_UNSUPPORTED, "column shape does not fit this plan's nx");
   if (pass < NUM_COL_OPS)
     p->colsel[pass] = shape;
-  if (pass == COL_RESID_PK) p->pk_asked = true;
-  if (pass >= NUM_COL_OPS)
+  else
     p->modesel[pass - NUM_COL_OPS] = shape;
   if (p->graph) {  // the captured iteration used the previous shapes
     cudaGraphExecDestroy(p->graph);
