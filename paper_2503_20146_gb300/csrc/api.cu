@@ -660,23 +660,28 @@ PassArgs colq_args(const pwf_plan* p, PassArgs a, int which, int conj) {
 // row pass on axis x, column pass on axis y
 // PWF_FLAG_CHECK_FINITE: after every pass a scan of what it wrote; the first
 // pass (in stream order) whose output holds a NaN or an infinity leaves its id
-__global__ void k_scan_finite(const float* v, size_t n, int id, int* word) {
+// (values in rows of `len`, `stride` apart).
+__global__ void k_scan_finite(const float* v, size_t n, size_t len, size_t stride, int id, int* word) {
   bool bad = false;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    bad |= !isfinite(v[i]);
+    bad |= !isfinite(v[len == stride ? i : i / len * stride + i % len]);
   if (__syncthreads_or(bad) && threadIdx.x == 0) atomicCAS(word, -1, id);
 }
 
-cudaError_t scan_output(pwf_plan* p, const char* name, const void* ptr, int proj0, int nproj, int floats_per_px) {
+// packed: only the packed rows, which sit on the even rows of a complex field
+// (the others are not written)
+cudaError_t scan_output(pwf_plan* p, const char* name, const void* ptr, int proj0, int nproj, int floats_per_px,
+                        bool packed = false) {
   if (!p->scan_word || !ptr) return cudaSuccess;
   int id = 0;
   while (id < (int)p->scan_names.size() && std::strcmp(p->scan_names[id], name) != 0) id++;
   if (id == (int)p->scan_names.size()) p->scan_names.push_back(name);
   const size_t px = (size_t)p->d.ny * p->d.nx;
   const float* v = static_cast<const float*>(ptr) + (size_t)proj0 * px * floats_per_px;
-  const size_t n = (size_t)nproj * px * floats_per_px;
+  const size_t n = (size_t)nproj * px * floats_per_px / (packed ? 2 : 1);
+  const size_t len = (size_t)p->d.nx * floats_per_px, stride = packed ? 2 * len : len;
   return enqueue(p, "scan_finite", [&] {
-    k_scan_finite<<<grid_for(n), 256, 0, p->stream>>>(v, n, id, p->scan_word);
+    k_scan_finite<<<grid_for(n), 256, 0, p->stream>>>(v, n, len, stride, id, p->scan_word);
     return cudaGetLastError();
   });
 }
@@ -701,8 +706,9 @@ const char* const kPkRowNames[NUM_PKROW_OPS] = {"row_real_fft_pk", "row_real_out
 cudaError_t row_pk(pwf_plan* p, int op, PassArgs a, int nproj) {
   a = row_args(p, a);
   cudaError_t e = enqueue(p, kPkRowNames[op], [&] { return p->krow->row_pk[op](a, nproj, p->stream); });
-  if (e == cudaSuccess && op == PKROW_OUT) e = scan_output(p, kPkRowNames[op], a.f_out, a.proj0, nproj, 1);
-  return e;
+  if (e != cudaSuccess) return e;
+  return op == PKROW_OUT ? scan_output(p, kPkRowNames[op], a.f_out, a.proj0, nproj, 1)
+                         : scan_output(p, kPkRowNames[op], a.out, a.proj0, nproj, 2, true);
 }
 // the column-axis twiddles of the radix schedule a column shape was built with
 PassArgs sched_tables(const pwf_plan* p, PassArgs a, int sched) {
@@ -721,7 +727,8 @@ cudaError_t col(pwf_plan* p, int op, PassArgs a, int nproj) {
 cudaError_t col_iotf_pk(pwf_plan* p, PassArgs a, int nproj) {
   const ColVariant& v = p->kcol->iotf_pk[p->colsel[COL_RESID_PK]];
   a = sched_tables(p, col_args(p, a), v.sched);
-  return enqueue(p, "col_iotf_pk", [&] { return v.launch(a, nproj, p->stream); });
+  cudaError_t e = enqueue(p, "col_iotf_pk", [&] { return v.launch(a, nproj, p->stream); });
+  return e != cudaSuccess ? e : scan_output(p, "col_iotf_pk", a.out, a.proj0, nproj, 2, true);
 }
 cudaError_t col_q(pwf_plan* p, PassArgs a, int which, int conj, int nproj) {
   a = sched_tables(p, colq_args(p, a, which, conj), p->kcol->colv[COL_Q][p->colsel[COL_Q]].sched);
