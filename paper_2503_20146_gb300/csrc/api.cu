@@ -971,9 +971,8 @@ bool packed_resid(const pwf_plan* p) {
 //                   2 x 2048^2      264 / 238  579 / 527
 // At the line itself the two differ by up to 7 % either way, by no rule on
 // lengths, tiles or batch; from 2^22 on the packed form is never slower.
-bool packed_real(const pwf_plan* p) {
-  return packed_resid(p) && (long long)p->d.batch * p->d.ny * p->d.nx >= 1ll << 20;
-}
+bool packed_size(const pwf_plan_desc& d) { return (long long)d.batch * d.ny * d.nx >= 1ll << 20; }
+bool packed_real(const pwf_plan* p) { return packed_resid(p) && packed_size(p->d); }
 
 // one fused iteration (or the body of pwf_step): X must hold F_row{exp psi}
 pwf_status fused_iteration(pwf_plan* p, pwf_state* st, const float* y, const float2* t, float2* psi,
@@ -1510,8 +1509,10 @@ pwf_status pwf_plan_create(const pwf_plan_desc* desc, pwf_plan** out) {
     pwf_plan_destroy(p);
     return PWF_ERR_CUDA;
   }
+  const bool with_pk = packed_size(d);  // the packed real passes are prepared for the plans that may run them
   for (int op = 0; op < NUM_ROW_OPS; op++)
-    if (p->krow->row_prep[op]() != cudaSuccess || (op < NUM_PKROW_OPS && p->krow->row_pk_prep[op]() != cudaSuccess)) {
+    if (p->krow->row_prep[op]() != cudaSuccess ||
+        (with_pk && op < NUM_PKROW_OPS && p->krow->row_pk_prep[op]() != cudaSuccess)) {
       cudaGetLastError();
       pwf_plan_destroy(p);
       return PWF_ERR_CUDA;
@@ -1525,7 +1526,8 @@ pwf_status pwf_plan_create(const pwf_plan_desc* desc, pwf_plan** out) {
       }
   for (int op = 0; op < NUM_COL_OPS; op++)
     for (int v = 0; v < p->kcol->ncolv[op]; v++)
-      if (p->kcol->colv[op][v].prep() != cudaSuccess || (op == COL_RESID_PK && p->kcol->iotf_pk[v].prep() != cudaSuccess)) {
+      if (p->kcol->colv[op][v].prep() != cudaSuccess ||
+          (with_pk && op == COL_RESID_PK && p->kcol->iotf_pk[v].prep() != cudaSuccess)) {
         cudaGetLastError();
         pwf_plan_destroy(p);
         return PWF_ERR_CUDA;

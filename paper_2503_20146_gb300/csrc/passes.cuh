@@ -2000,7 +2000,11 @@ template <int N, int OP>
 void add_col_op(LengthKernels& k) {
   // first entry = default before tuning. Left out where they never came near the
   // fastest: transposed tiles and 4-column TMA tiles from length 1024 on, wide
-  // tiles with 32 values per thread (they spill).
+  // tiles with 32 values per thread (they spill), and single-buffered tiles of one
+  // column per thread below length 1024 (best there: level with the fastest shape
+  // on fields of one wave, 5 % to 50 % behind on larger ones; fastest at 1024) and
+  // with 4 columns or the alternative schedule (8 % to 60 % behind everywhere).
+  // Every shape costs each plan some 30 us to prepare and time.
   constexpr bool LONG = N >= 1024, WIDE = ept_for(N) >= 32;
   constexpr int FIRST = !WIDE ? 0 : OP == COL_PRECOND_REG ? 1 : OP == COL_RESID_IOTF2 ? 2 : 0;
   if constexpr (FIRST == 1) add_col_variant<N, OP, 4, 0>(k);
@@ -2021,8 +2025,7 @@ void add_col_op(LengthKernels& k) {
   add_col_variant<N, OP, 4, 4>(k);
   add_col_variant<N, OP, 8, 5>(k);
   if constexpr (!LONG) add_col_variant<N, OP, 4, 5>(k);
-  add_col_variant<N, OP, 8, 7>(k);
-  add_col_variant<N, OP, 4, 7>(k);
+  if constexpr (LONG) add_col_variant<N, OP, 8, 7>(k);
 }
 
 // the radices of this translation unit's schedule of length N into slot `set`
@@ -2049,7 +2052,6 @@ void add_schedule_shapes(LengthKernels& k) {
     add_col_variant<N, OP, 8, 1>(k);
     add_col_variant<N, OP, 16, 0>(k);
     add_col_variant<N, OP, 8, 0>(k);
-    add_col_variant<N, OP, 8, 7>(k);
   };
   op_shapes(std::integral_constant<int, COL_Q>{});
   op_shapes(std::integral_constant<int, COL_IOTF>{});
