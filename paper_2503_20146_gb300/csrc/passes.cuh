@@ -132,15 +132,18 @@ __device__ __forceinline__ float2 cexpf2(float2 z) {
   return make_float2(m * c, m * s);
 }
 
-// sin and cos to within an ulp without a slow path in the common range: the
-// phase is reduced by multiples of pi/2 (Cody-Waite, C1 + C2 = pi/2 to 2^-48,
-// one FMA each, so that k <= 2^16 turns leave 2^-33), then odd and even
-// polynomials on [-pi/4, pi/4] (minimax fits of (sin r - r)/r^3 and
-// (cos r - 1 + r^2/2)/r^4 in r^2, weighted for relative error: 2^-27.9 and
-// 2^-33). Against the library sincosf this removes the branch to its
-// large-argument code, which kept the loads of a thread's values from being
-// issued together. Phases beyond 65536 rad take the library routine (out of
-// line: inlined at every value it overflows the instruction cache).
+// sin and cos without a slow path in the common range, to 1.2 2^-24 of the unit
+// circle (absolute: near their zeros at large phases that is many ulp of a small
+// result, which exp(psi) adds to a component near 1). The phase is reduced by
+// multiples of pi/2 (Cody-Waite, C1 + C2 = pi/2 to 2^-48, one FMA each: the
+// reduced phase is off by two roundings, and by 2^-33 after 2^15 quarter turns),
+// then odd and even polynomials on [-pi/4, pi/4] (minimax fits of (sin r - r)/r^3
+// and (cos r - 1 + r^2/2)/r^4 in r^2, weighted for relative error: 2^-27.9 and
+// 2^-33). Rms error 0.29 2^-24, modulus right to 4e-10 on average. Against the
+// library sincosf this removes the branch to its large-argument code, which kept
+// the loads of a thread's values from being issued together. Phases beyond 65536
+// rad take the library routine (out of line: inlined at every value it
+// overflows the instruction cache).
 static __device__ __noinline__ float2 sincos_big(float y) {
   float2 r;
   sincosf(y, &r.x, &r.y);
@@ -169,12 +172,12 @@ __device__ __forceinline__ void sincos_acc(float y, float& s, float& c) {
   }
 }
 
-// exp(z) to about one ulp, for the object field x = exp(psi) that enters the
-// forward model and the gradient. The hardware approximations of cexpf2 are
-// 2^-21.4 absolute on the phase and a few ulp on the modulus; both errors are
-// smooth functions of psi, so over a smooth object they add up coherently in
-// the lowest spatial frequencies of the modelled intensity, where the
-// preconditioner of Eq. (11) amplifies them by up to N^2. cexpf2 stays where
+// exp(z) to about 2^-24 of its modulus, for the object field x = exp(psi) that
+// enters the forward model and the gradient. The hardware approximations of
+// cexpf2 are 2^-21.4 absolute on the phase and a few ulp on the modulus; both
+// errors are smooth functions of psi, so over a smooth object they add up
+// coherently in the lowest spatial frequencies of the modelled intensity, where
+// the preconditioner of Eq. (11) amplifies them by up to N^2. cexpf2 stays where
 // its errors cancel: the correlation sums.
 __device__ __forceinline__ float2 cexpf_acc(float2 z) {
   float s, c;
