@@ -17,7 +17,6 @@
 #include <vector>
 
 #include "../../include/pwf.h"
-#include "host_tables.h"
 #include "persist.cuh"
 
 namespace pwf {

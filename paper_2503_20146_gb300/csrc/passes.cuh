@@ -34,9 +34,6 @@ __host__ __device__ constexpr size_t row_smem_bytes(int n) {
   return (size_t)rows_for(n) * row_smem_len(n) * sizeof(float2);
 }
 
-
-
-
 // Barrier of the two rows 2y', 2y' + 1 of a row-pass CTA (the packed passes):
 // the warp when both fit in one, else named barrier 8 + pair over their
 // 2 TPF threads (rows use ids 1..4 only when TPF > 32, so these stay clear).
@@ -590,24 +587,24 @@ __global__ void __launch_bounds__(row_threads(N), row_min_blocks(N, OP)) row_ker
 // Row passes whose fields are real on the real-space side: one transform per
 // packed row y' (rows 2y' and 2y' + 1 of the field as real and imaginary part),
 // so half the transforms and 4 bytes per pixel of spectrum instead of 8. The
-// TPF threads of a packed row hold both rows; packed rows past the last one
-// (a CTA may hold more than are left) repeat it and store nothing.
+// TPF threads of a packed row hold both rows. A CTA's packed rows belong to one
+// projection: column lengths with packed shapes have a multiple of 16 of them,
+// and ROWS is a power of two up to 16 (launch_row_pk checks).
 template <int N, int OP>
-__global__ void __launch_bounds__(row_threads(N), row_min_blocks(N, ROW_FFT)) row_pk_kernel(const PassArgs a, int nrows) {
+__global__ void __launch_bounds__(row_threads(N), row_min_blocks(N, ROW_FFT)) row_pk_kernel(const PassArgs a) {
   pdl_wait();
   constexpr int EPT = ept_for(N), TPF = tpf_for(N), ROWS = rows_for(N);
   constexpr int RS = first_radix<N, FWD>();
   constexpr int RK = last_radix<N, FWD>();
   extern __shared__ float2 smem[];
   const int rr = threadIdx.x / TPF, t = threadIdx.x - rr * TPF;
-  int row = blockIdx.x * ROWS + rr;
-  const bool valid = row < nrows;
-  row = (valid ? row : nrows - 1) + a.proj0 * (a.ny / 2);
-  const int proj = row / (a.ny / 2);
-  if (skip_proj(a, proj)) return;
+  const long long row = (long long)blockIdx.x * ROWS + rr + (long long)a.proj0 * (a.ny / 2);
+  const int proj = (int)(row / (a.ny / 2));
+  if (skip_proj(a, proj)) return;  // uniform per CTA
   const size_t rb = 2 * (size_t)row * N;  // the even row
   const RowLayout<N, ROWS * TPF> sm{smem + rr * row_smem_len(N), 1 + rr};
   float2 v[EPT];
+  float part[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
   if constexpr (OP == PKROW_FFT) {
 #pragma unroll
     for (int j = 0; j < EPT; j++) {
@@ -620,38 +617,27 @@ __global__ void __launch_bounds__(row_threads(N), row_min_blocks(N, ROW_FFT)) ro
     fft_run<N, INV>(v, sm, t, a.tw_inv);
   }
   if constexpr (OP == PKROW_OUT) {
-    if (valid) {
 #pragma unroll
-      for (int j = 0; j < EPT; j++) {
-        const size_t o = rb + slot_index<N, RS>(t, j);
-        a.f_out[o] = v[j].x;
-        a.f_out[o + N] = v[j].y;
-      }
+    for (int j = 0; j < EPT; j++) {
+      const size_t o = rb + slot_index<N, RS>(t, j);
+      a.f_out[o] = v[j].x;
+      a.f_out[o + N] = v[j].y;
     }
     return;
   }
   if constexpr (OP == PKROW_RESID) {
-    float part = 0.f;
 #pragma unroll
     for (int j = 0; j < EPT; j++) {
       const size_t o = rb + slot_index<N, RS>(t, j);
       const float e0 = a.y[o] - v[j].x, e1 = a.y[o + N] - v[j].y;
-      part = fmaf(e0, e0, fmaf(e1, e1, part));
+      part[0] = fmaf(e0, e0, fmaf(e1, e1, part[0]));
       v[j] = make_float2(-e0, -e1);
     }
-    // a CTA may hold rows of two projections: each row adds its own sum
-    constexpr int W = TPF < 32 ? TPF : 32;
-    double d = valid ? (double)part : 0.0;
-    const unsigned mask = ROWS * TPF >= 32 ? 0xffffffffu : ((1u << (ROWS * TPF & 31)) - 1u);
-#pragma unroll
-    for (int o = W / 2; o > 0; o >>= 1) d += __shfl_xor_sync(mask, d, o);
-    if (valid && t % W == 0) atomicAdd(&a.acc[(size_t)proj * NACC + ACC_LOSS], d);
   }
   fft_run<N, FWD>(v, sm, t, a.tw_fwd);
-  if (valid) {
 #pragma unroll
-    for (int j = 0; j < EPT; j++) a.out[rb + pk_pos<N>(slot_index<N, RK>(t, j))] = v[j];
-  }
+  for (int j = 0; j < EPT; j++) a.out[rb + pk_pos<N>(slot_index<N, RK>(t, j))] = v[j];
+  if constexpr (OP == PKROW_RESID) block_reduce_add<1>(part, a.acc, proj * NACC + ACC_LOSS, smem);
 }
 
 // ---------------------------------------------------------------------------
@@ -789,6 +775,10 @@ __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(gsrc) : "memory");
 }
+__device__ __forceinline__ void cp_async8(void* smem_dst, const void* gsrc) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(gsrc) : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int K>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(K) : "memory"); }
@@ -913,17 +903,6 @@ __global__ void __launch_bounds__(col_threads(N, C), col_min_blocks_op<OP>(col_t
   cp_async_wait<0>();
 }
 
-// Transposed tile: the prefetch (8-byte cp.async) stores each of the C columns
-// contiguously in shared memory (column stride S, S = 4 mod 16 slots, so the
-// row-major copy pattern of a warp - C columns x 32/C rows - falls on every
-// bank pair exactly twice), the TPF threads of one column run its transforms
-// exactly like a row pass with a barrier of their own, and the results go
-// back through shared memory so that the global stores are row-major and
-// coalesced. Single-input ops only.
-__device__ __forceinline__ void cp_async8(void* smem_dst, const void* gsrc) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(gsrc) : "memory");
-}
 __host__ __device__ constexpr int colt_stride(int n) {
   return row_smem_len(n) + ((4 - row_smem_len(n) % 16) + 16) % 16;
 }
@@ -1474,10 +1453,13 @@ __global__ void __launch_bounds__(col2_threads(N, C), col2_min_blocks(N, C)) col
   }
 }
 
-// The TMA map of a batch of complex64 fields [B][ny][nx] seen as float32
-// [B][ny][2 nx]: box = 2C floats (C columns) x min(ny, 256) rows x 1 field.
-// Encoded on the host through the driver entry point (no libcuda link).
-
+// Transposed tile: the prefetch (8-byte cp.async) stores each of the C columns
+// contiguously in shared memory (column stride S, S = 4 mod 16 slots, so the
+// row-major copy pattern of a warp - C columns x 32/C rows - falls on every
+// bank pair exactly twice), the TPF threads of one column run its transforms
+// exactly like a row pass with a barrier of their own, and the results go
+// back through shared memory so that the global stores are row-major and
+// coalesced. Single-input ops only.
 template <int N, int OP, int C>
 __global__ void __launch_bounds__(col_threads(N, C), col_min_blocks(col_threads(N, C), ept_for(N)))
     col_kernel_t(const PassArgs a, int nproj) {
@@ -1541,7 +1523,6 @@ __global__ void __launch_bounds__(col_threads(N, C), col_min_blocks(col_threads(
     float2 v[EPT];
     float2 s2[1];
     float part[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-    int RO;  // slot radix of the results
     if constexpr (OP == COL_IFFT) {
 #pragma unroll
       for (int j = 0; j < EPT; j++) v[j] = cscale(sm[slot_index<N, RK>(t, j)], a.scale);
@@ -1561,7 +1542,6 @@ __global__ void __launch_bounds__(col_threads(N, C), col_min_blocks(col_threads(
 #pragma unroll
       for (int j = 0; j < EPT; j++) sm[slot_index<N, RS>(t, j)] = v[j];
     }
-    (void)RO;
     __syncthreads();
 #pragma unroll 8
     for (int kk = 0; kk < ELEMS / NT; kk++) {
@@ -1765,9 +1745,10 @@ cudaError_t prep_row_pk() {
 template <int N, int OP>
 cudaError_t launch_row_pk(const PassArgs& a, int nproj, cudaStream_t s) {
   constexpr int ROWS = rows_for(N);
-  const int nrows = nproj * (a.ny / 2);
-  return launch_pass(row_pk_kernel<N, OP>, dim3((unsigned)((nrows + ROWS - 1) / ROWS)), dim3(row_threads(N)),
-                     row_smem_bytes(N), s, a.pdl, a, nrows);
+  if ((a.ny / 2) % ROWS != 0) return cudaErrorInvalidValue;
+  const long long nrows = (long long)nproj * (a.ny / 2);
+  return launch_pass(row_pk_kernel<N, OP>, dim3((unsigned)(nrows / ROWS)), dim3(row_threads(N)), row_smem_bytes(N), s,
+                     a.pdl, a);
 }
 
 // column-pass shape variants: tile width C, pipelined or not
@@ -1890,7 +1871,7 @@ template <int N, int C, bool RES>
 int PkShape<N, C, RES>::resident = 1;
 
 // whole warps (the output pairs rows by shuffle), even chunk split; a plan
-// takes a shape only where C divides nx/2 (pk_fits)
+// takes a shape only where C divides nx/2 (shape_fits)
 template <int N, int C>
 constexpr bool pk_shape_ok() {
   constexpr int th = col2_threads(N, C);
@@ -2094,7 +2075,10 @@ LengthKernels make_length_kernels() {
   add_col_op<N, COL_PRECOND_REG>(k);
   add_col_op<N, COL_FFT>(k);
   add_col_op<N, COL_IFFT>(k);
-  add_pk_variant<N, 8>(k);  // first entry = default before tuning (fits every nx >= 16)
+  // first entry = default before tuning: 8 positions, which fit every nx; lengths 32
+  // and 96 have only the 16-position shape, which nx = 16 does not hold (such a plan
+  // takes the full complex form), and length 16 none
+  add_pk_variant<N, 8>(k);
   add_pk_variant<N, 4>(k);
   if constexpr (ept_for(N) < 32) add_pk_variant<N, 16>(k);
   static_assert(mode_shape_ok<N, CM_FWD, 16, false>() || mode_shape_ok<N, CM_FWD, 8, false>() ||
