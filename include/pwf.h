@@ -102,11 +102,10 @@ typedef struct pwf_state pwf_state;
                                     square grids of 64, 128, 256 or 512 only, else
                                     PWF_ERR_UNSUPPORTED. At most one of PERSISTENT,
                                     GRAPH and CLUSTER (else PWF_ERR_INVALID_ARG).
-                                    With none of the three, a plan takes this
-                                    solver where it measured faster: square
-                                    128^2 IOTF/coherent plans whose batch one
-                                    wave of clusters holds (not with
-                                    PWF_FLAG_CHECK_FINITE)                         */
+                                    With none of the three, the plans that take
+                                    this solver are the square 128^2 IOTF/coherent
+                                    ones whose batch one wave of clusters holds
+                                    (not with PWF_FLAG_CHECK_FINITE)               */
 #define PWF_FLAG_CHECK_FINITE 0x200u /* debug: after every pass a scan of what it
                                     wrote; pwf_state_read (and pwf_solve) then
                                     return PWF_ERR_NONFINITE naming, in

@@ -1550,12 +1550,15 @@ pwf_status pwf_plan_create(const pwf_plan_desc* desc, pwf_plan** out) {
       pwf_plan_destroy(p);
       return PWF_ERR_UNSUPPORTED;
     }
-    // With no solver asked for, the cluster-resident solver takes the plans it
-    // measured faster on: lengths with its one-warp-per-transform schedule
-    // (128^2: 50 against 58 us per iteration, IOTF), batches that one wave of
-    // clusters holds (9 x 128^2 needed two waves: 99 against 58 us).
+    // With no solver asked for, the cluster-resident solver takes square plans of up
+    // to 128^2 with its one-warp-per-transform schedule whose batch one wave of
+    // clusters holds. us per iteration, cluster / graph: 128^2 coherent 42 / 43,
+    // IOTF 48 / 48 (one launch in place of a graph with a loop, and level in time),
+    // 8 x 128^2 83 / 43 (two waves). 256^2, which has such a schedule too, stays
+    // with the graph, 88 / 51 and 103 / 58: a pass of four times the work keeps one
+    // cluster's SMs busy for longer than the graph's gaps between passes.
     const bool no_solver = !(d.flags & (PWF_FLAG_PERSISTENT | PWF_FLAG_GRAPH | PWF_FLAG_CLUSTER));
-    const bool try_cluster = eligible && no_solver && !(d.flags & PWF_FLAG_CHECK_FINITE) &&
+    const bool try_cluster = eligible && no_solver && !(d.flags & PWF_FLAG_CHECK_FINITE) && d.nx <= 128 &&
                              p->kcol->persist_cluster[1] != nullptr && p->ax.tw_fwd_alt && p->ay.tw_fwd_alt;
     if ((d.flags & PWF_FLAG_CLUSTER) || try_cluster) {
       if ((r = dalloc(p, &p->gpart, (size_t)d.batch * PERSIST_MAX_CLUSTER * NACC)) ||
