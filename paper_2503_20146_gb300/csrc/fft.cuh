@@ -391,12 +391,11 @@ struct Sched {
 };
 
 // The alternative schedules (set 1): the same stages in another order where
-// that keeps the values per thread, or smaller radices where it cuts them (1024
-// with 16 instead of 32 values)
-// (fewer registers per transform, more warps per SM, shorter dependent chains
-// per thread, at the price of more exchanges: 128 = 4.4.4.2 runs one
-// transform per warp with four values per thread; 768 and 1536 keep 12 values
-// per thread instead of 24).
+// that keeps the values per thread, or smaller radices where it cuts them: fewer
+// registers per transform, more warps per SM, shorter dependent chains per
+// thread, at the price of more exchanges (128 = 4.4.4.2 runs one transform per
+// warp with four values per thread; 768 and 1536 keep 12 values per thread
+// instead of 24, 1024 16 instead of 32).
 __host__ __device__ constexpr Sched sched_alt(int n) {
   switch (n) {
     case 128: return {128, 4, 4, 4, 4, 2, 1, 1};
@@ -530,7 +529,10 @@ __host__ __device__ constexpr int col_tile_rows(int n, int c) { return col_padde
 // Column transforms in two-wide instructions (fewer issue slots, but the pairs
 // tie registers together) or scalar ones: two-wide where a thread holds 32
 // values (COL_Q as column pairs at 1024, 32.32: 0.764 ms against 0.843 scalar;
-// 16.8.8: 0.855 against 0.815).
+// 16.8.8: 0.855 against 0.815). With 24 values they differ by pass, two-wide /
+// scalar on 32 x 768^2: COL_Q 0.100 / 0.096, COL_RESID_PK 0.090 / 0.095,
+// COL_PRECOND_REG 0.212 / 0.205; on 8 x 1536^2 0.123 / 0.117, 0.118 / 0.120, 0.283 /
+// 0.300: an iteration has four COL_Q and one of each other, so scalar.
 __host__ __device__ constexpr bool col_packed(int n) { return ept_for(n) >= 32; }
 template <int N, int C>
 struct ColLayout {

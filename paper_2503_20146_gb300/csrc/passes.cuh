@@ -249,7 +249,9 @@ __device__ __forceinline__ void row_body(const PassArgs& a, long long row, int t
   // the compiler knows, which would leave one load in flight at a time. On 180
   // x 1024^2 (ms per launch): row_grad_pack 1.78 -> 1.18, row_nesterov_fft 2.04
   // -> 1.72; on 24 x 1024^2 row_mode_int 0.162 -> 0.094, col_mode_back 0.187 ->
-  // 0.139, row_exp_fft 0.211 -> 0.072 (with sincos_acc).
+  // 0.139, row_exp_fft 0.211 -> 0.072 (with sincos_acc). Groups of 4 / 8 / all,
+  // row_grad_pack: 16 x 2048^2 0.541 / 0.492 / 0.512, 8 x 1536^2 0.256 / 0.254 / 0.265,
+  // 32 x 768^2 0.199 / 0.195 / 0.209, 64 x 512^2 0.123 / 0.122 / 0.121.
   constexpr int BL = EPT % 8 == 0 ? 8 : EPT;
 
   // Pull this row's side inputs into L2 while the first transform runs.
@@ -437,7 +439,10 @@ __device__ __forceinline__ void row_body(const PassArgs& a, long long row, int t
     }
   } else if constexpr (OP == ROW_NESTEROV_FFT || OP == ROW_NESTEROV) {
     const float beta = *a.beta;
-    constexpr int BN = EPT >= 32 ? 8 : EPT % 4 == 0 ? 4 : EPT;  // three side inputs: what the registers hold
+    // three side inputs, in groups that the registers hold: 4, or 8 with 32 values
+    // per thread (180 x 1024^2 1.745 -> 1.719 ms). 8 elsewhere costs: 16 x 2048^2 0.625 ->
+    // 0.646, 8 x 1536^2 0.232 -> 0.249, 64 x 512^2 0.162 -> 0.174, 64 x 256^2 0.048 -> 0.059.
+    constexpr int BN = EPT >= 32 ? 8 : EPT % 4 == 0 ? 4 : EPT;
 #pragma unroll
     for (int j0 = 0; j0 < EPT; j0 += BN) {
      float2 ps[BN], ph[BN];
