@@ -1552,8 +1552,8 @@ pwf_status pwf_plan_create(const pwf_plan_desc* desc, pwf_plan** out) {
     }
     // With no solver asked for, the cluster-resident solver takes square plans of up
     // to 128^2 with its one-warp-per-transform schedule whose batch one wave of
-    // clusters holds. us per iteration, cluster / graph: 128^2 coherent 42 / 43,
-    // IOTF 48 / 48 (one launch in place of a graph with a loop, and level in time),
+    // clusters holds. us per iteration, cluster / graph: 128^2 coherent 42 / 38 to 44
+    // (by the tuner's picks), IOTF 48 / 48 (one launch in place of a graph with a loop),
     // 8 x 128^2 83 / 43 (two waves). 256^2, which has such a schedule too, stays
     // with the graph, 88 / 51 and 103 / 58: a pass of four times the work keeps one
     // cluster's SMs busy for longer than the graph's gaps between passes.
