@@ -1540,8 +1540,8 @@ pwf_status pwf_plan_create(const pwf_plan_desc* desc, pwf_plan** out) {
   }
   // persistent solver (PWF_FLAG_PERSISTENT): square IOTF/coherent plans of
   // the built sizes. Not the default: on a GB300 its grid barriers cost more
-  // than the graph replay's launch gaps at every size it serves (128^2: 132
-  // against 56 us per iteration; 512^2: 180 against 80)
+  // than the graph replay's launch gaps at every size it serves (128^2: 111
+  // against 38 us per iteration; 512^2: 156 against 69)
   {
     const bool eligible = p->kcol->persist != nullptr && d.nx == d.ny && p->modes.empty() &&
                           !(d.flags & PWF_FLAG_PLAIN);
